@@ -316,8 +316,8 @@ LB_RD_API int lb_rd_batch_set_graph(lb_rd_batch *b, int32_t steps_per_graph);
 /* Time steps per launch, 1 .. 8: 2 runs the two-step (temporal blocking)
  * kernel over all instances, bitwise the same as two single steps, when the
  * instances are FP32 with two state copies and nx a multiple of 256; other
- * values >= 2 (and 2 otherwise) run the depth-K kernel over the (band, strip)
- * units of all instances (FP32, two state copies, any nx; bitwise the same as
+ * values >= 2 (and 2 otherwise) run the depth-K kernel over the rows of all
+ * instances (FP32, two state copies, any nx; bitwise the same as
  * K single steps; for K <= 5 (D2Q9) or 6 (D2Q5) its form with two columns per
  * lane; the default for such batches: 5 for D2Q9, 6 for D2Q5); 16-bit
  * deviation storage runs its own depth-K kernels, K = 2 .. 5 (the

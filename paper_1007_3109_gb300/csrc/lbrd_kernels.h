@@ -162,12 +162,12 @@ int batch_tb2_strip();
 cudaError_t launch_batch_tb2(const TbwItem *items, int n, int64_t total_units, int Q, int S, cudaStream_t st);
 // Batched K-step launches (K = 2 .. 8; FP32, two state copies): the depth-K
 // kernel over the (band, strip) units of a list of grids (for K <= 5 (D2Q9)
-// or 6 (D2Q5) its two-column form).  Item k's units
+// or 6 (D2Q5) its two-column form).  The one-column form's units of item k
 // are [unit_begin, unit_begin + nstrips * ceil(ny / band)), strips of the
-// kernel's output columns (34 - 2K, or 64 - 2 HL) fastest.  batch_deep_plan
-// fills nstrips and band of every item (one band height in rows for the whole
-// list, chosen for the launch's warp count) and returns the total unit count,
-// or -1 for an unsupported K.  v16: every grid has nx
+// kernel's 34 - 2K output columns fastest; the two-column form shares out the
+// list's rows (list_rows.cuh).  batch_deep_plan fills the descriptors (one-column
+// form: one band height in rows for the whole list, chosen for the launch's warp
+// count) and returns the total unit (row) count, or -1 for an unsupported K.  v16: every grid has nx
 // and pitch multiples of 4 (16-byte staging).  emit: the launch also writes
 // rho(t + K) of every item to its a.rho_out (the last launch of a call).
 // rk: the reaction kind that every item has (a.rkind), or -1 when they differ
@@ -175,6 +175,8 @@ cudaError_t launch_batch_tb2(const TbwItem *items, int n, int64_t total_units, i
 struct DeepItem {
     StepArgs a;
     int64_t unit_begin, nstrips, band;
+    int64_t run_strips, next;  // two-column kernels: the list's rows (list_rows.cuh)
+    int gs, lockstep;
 };
 // The same over 16-bit deviation storage (K = 2 .. 5; half_kind 0 bf16, 1 fp16;
 // any nx a multiple of 4): the two-column depth-K kernel of

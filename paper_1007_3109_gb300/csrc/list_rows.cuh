@@ -1,0 +1,132 @@
+// Division of a list of grids among the warps of a depth-K launch, by rows.
+//
+// The two-column depth-K kernels walk strips of columns down rows.  Over a list
+// the work is one line of rows: strip after strip, every strip its grid's ny
+// rows, cut into equal parts, one per worker.  A worker walks its part
+// segment by segment (a segment ends with its strip), paying the 2K rows that
+// fill the levels once per segment.
+//
+// A worker is a block, whose NW warps walk NW adjacent strips side by side
+// (group size NW), or a warp (group size 1).  Strips of consecutive grids of
+// equal shape (a "run") are numbered through, so a group may hold the last
+// strips of one grid and the first of the next; the last group of a run may be
+// partly empty, its remaining warps idle.  Blocks keep the accesses of their
+// warps together (the halo columns two strips share are read at about the same
+// time, and DRAM sees longer contiguous pieces); single warps lose nothing to
+// partly empty groups in lists of uneven grids.
+#pragma once
+
+#include "lbrd_kernels.h"
+
+namespace lbrd {
+
+namespace {
+
+// Sites of a list above which the warps of a block meet every four rows (FP32
+// D2Q9): the halo columns that two strips share are then read while they are in
+// L2.  40 uneven grids of sides up to 2048 (60 M sites): 422 -> 388 us per
+// step; 256 grids of 255^2: 137 -> 127; 256^2: no change.  Lists that sit
+// closer to L2 lose a little instead (9 x 512^2, 2.4 M sites: 16.7 -> 17.3).
+constexpr int64_t kLockstepSites = 8 << 20;
+
+// A cut of the line moved to the end of a strip that is at most `slack` rows
+// away, so that no worker fills the levels for a few rows of a strip.
+__device__ __forceinline__ int64_t list_rows_snap(const DeepItem *__restrict__ items, int nitems, int64_t u,
+                                                  int64_t total, int slack, int &run) {
+    if (u <= 0 || u >= total) return u;
+    for (int nx = (int)items[run].next; nx < nitems && items[nx].unit_begin <= u; nx = (int)items[run].next) run = nx;
+    const int ny = (int)items[run].a.ny;
+    const int at = (int)((u - items[run].unit_begin) % ny);
+    return at <= slack ? u - at : (ny - at <= slack ? u + (ny - at) : u);
+}
+
+// A warp's place in the line: its rows [u, u_end), the run of row u and the
+// group size.  Held in shared memory, one per warp, so that it takes no
+// registers while a segment's rows are walked.
+struct ListWalk {
+    int64_t u, u_end;
+    int run, gs;
+};
+
+// The place where this warp starts (called by one lane).
+template <int NW, int K>
+__device__ __forceinline__ void list_rows_begin(const DeepItem *__restrict__ items, int nitems, int64_t total, int w,
+                                                ListWalk &walk) {
+    const int gs = (int)items[0].gs;
+    const int64_t worker = gs == 1 ? (int64_t)blockIdx.x * NW + w : blockIdx.x;
+    const int64_t nworkers = gs == 1 ? (int64_t)gridDim.x * NW : gridDim.x;
+    const int64_t rows = total / nworkers;
+    const int slack = rows + 1 < 2 * K ? (int)(rows + 1) / 2 : K;
+    int run = 0;
+    walk.u = list_rows_snap(items, nitems, total * worker / nworkers, total, slack, run);
+    walk.run = run;
+    walk.gs = gs;
+    walk.u_end = list_rows_snap(items, nitems, total * (worker + 1) / nworkers, total, slack, run);
+}
+
+// The next segment: rows [y0, y0 + ly) of strip `strip` of grid `item`;
+// `together`: every warp of the block walks a strip of it and the plan asks for
+// barriers (block-uniform).  Returns 1, 0 if this warp has no strip in it, or -1 at the end of the part.
+// Called by all lanes of the warp.
+__device__ __forceinline__ int list_rows_next(const DeepItem *__restrict__ items, int nitems, int w, int lane,
+                                              ListWalk &walk, int &item, int &strip, int &y0, int &ly,
+                                              bool &together) {
+    const volatile ListWalk &wk = walk;
+    const int64_t u = wk.u, u_end = wk.u_end;
+    if (u >= u_end) return -1;
+    const int gs = wk.gs;
+    int run = wk.run;
+    for (int nx = (int)items[run].next; nx < nitems && items[nx].unit_begin <= u; nx = (int)items[run].next) run = nx;
+    const int ny = (int)items[run].a.ny, ns = (int)items[run].nstrips;
+    const int64_t local = u - items[run].unit_begin;
+    const int group = (int)(local / ny);
+    y0 = (int)(local - (int64_t)group * ny);
+    ly = ny - y0;
+    if (u_end - u < ly) ly = (int)(u_end - u);
+    __syncwarp();  // every lane has read the place
+    if (lane == 0) {
+        walk.u = u + ly;
+        walk.run = run;
+    }
+    __syncwarp();
+    together = items[0].lockstep && gs > 1 && group * gs + gs <= (int)items[run].run_strips;
+    const int s = gs == 1 ? group : group * gs + w;
+    if (s >= (int)items[run].run_strips) return 0;
+    item = run + s / ns;
+    strip = s - (item - run) * ns;
+    return 1;
+}
+
+// Fills the runs, the line of rows and the group size (1 or NW) of a list whose
+// strips are WO columns wide; returns the length of the line.
+inline int64_t plan_list_rows(DeepItem *items, int n, int WO, int NW) {
+    int64_t strip_rows = 0, group_rows = 0;
+    for (int i = 0; i < n;) {
+        int j = i + 1;
+        while (j < n && items[j].a.nx == items[i].a.nx && items[j].a.ny == items[i].a.ny) ++j;
+        const int64_t ns = (items[i].a.nx + WO - 1) / WO, total = ns * (j - i);
+        for (int k = i; k < j; ++k) {
+            items[k].nstrips = ns;
+            items[k].run_strips = total;
+            items[k].next = j;
+        }
+        strip_rows += total * items[i].a.ny;
+        group_rows += (total + NW - 1) / NW * items[i].a.ny;
+        i = j;
+    }
+    const int gs = group_rows * NW <= 2 * strip_rows ? NW : 1;
+    int64_t at = 0, planes = 0;
+    for (int i = 0; i < n; ++i) planes += items[i].a.plane;
+    for (int i = 0; i < n; i = (int)items[i].next) {
+        for (int k = i; k < items[i].next; ++k) {
+            items[k].gs = gs;
+            items[k].lockstep = planes > kLockstepSites;
+            items[k].unit_begin = at;
+        }
+        at += (items[i].run_strips + gs - 1) / gs * items[i].a.ny;
+    }
+    return at;
+}
+
+}  // namespace
+}  // namespace lbrd

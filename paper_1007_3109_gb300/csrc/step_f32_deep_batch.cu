@@ -88,6 +88,7 @@ int64_t plan_batch(DeepItem *items, int n) {
         ge = BatchShape<Q, S, K, V16>::get(&full);
     }
     if (ge != cudaSuccess) return -1;
+    if constexpr (pair) return plan_list_rows(items, n, WO, NW);
     for (int i = 0; i < n; ++i) items[i].nstrips = (items[i].a.nx + WO - 1) / WO;
     const int64_t h = choose_band_height(K, items, n, (int64_t)full * NW);
     int64_t units = 0;
@@ -105,8 +106,8 @@ cudaError_t launch_pair_list(const DeepItem *items, int n, int64_t total_units, 
     unsigned full = 0;
     cudaError_t e = PS::get(&full);
     if (e != cudaSuccess) return e;
-    const int64_t nwarps = (int64_t)full * PS::NW;
-    const unsigned grid = total_units < nwarps ? (unsigned)((total_units + PS::NW - 1) / PS::NW) : full;
+    // total_units rows, shared out over the whole grid (at least one row per block)
+    const unsigned grid = total_units < (int64_t)full ? (unsigned)total_units : full;
     step_pair_kernel<Q, S, K, PS::NW, PS::NS, PS::MINB, true, true, !V16, RK>
         <<<grid, PS::NW * 32, PS::smem, st>>>(StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
     return cudaGetLastError();

@@ -39,6 +39,7 @@
 // reduction are those of the one-column kernel.
 #pragma once
 
+#include "list_rows.cuh"
 #include "step_f32_deep_kernel.cuh"
 
 namespace lbrd {
@@ -143,31 +144,48 @@ __global__ void __launch_bounds__(NW * 32, MINB)
             return g;
         }
     };
+    // lists of two-species D2Q9 grids: the species of a site packed (1024 x 256^2 at K = 5 runs at
+    // 98 against 99.4 us per step and quarter, one 512^2 grid at 4.8 against 5.5; D2Q5 and single grids
+    // gain nothing)
+    auto collide = [](const SegArgs &cg, float(&f0)[S][Q], float(&f1)[S][Q], float(&rho0)[S], float(&rho1)[S]) {
+        if constexpr (BATCH && Q == 9 && S == 2) collide_pair_species<Q, RK>(cg, f0, f1, rho0, rho1);
+        else collide_pair<Q, S, RK>(cg, f0, f1, rho0, rho1);
+    };
     double acc[S];
 #pragma unroll
     for (int s = 0; s < S; ++s) acc[s] = 0.0;
     const int64_t nwarps = (int64_t)gridDim.x * NW;
-    const int64_t units = BATCH ? total_units : nstrips * nbands;
+    const int64_t units = nstrips * nbands;
     const int cch = lane & 15, cpar = lane >> 4;  // copy role: chunk, plane parity
-    int it = 0;
-    for (int64_t u = (int64_t)blockIdx.x * NW + w; u < units; u += nwarps) {
-        int64_t local = u, ns = nstrips, bh = band;
+    // BATCH: the warp's place in the list's rows, kept in shared memory like gs
+    __shared__ ListWalk walk_sh[BATCH ? NW : 1];
+    if constexpr (BATCH) {
+        if (lane == 0) list_rows_begin<NW, K>(items, nitems, total_units, w, walk_sh[w]);
+        __syncwarp();
+    }
+    for (int64_t u = (int64_t)blockIdx.x * NW + w; BATCH || u < units; u += nwarps) {
+        int64_t strip;
+        int y0, ly;
+        bool together = false;
         if constexpr (BATCH) {
-            while (it + 1 < nitems && items[it + 1].unit_begin <= u) ++it;
-            load_seg(items[it].a, g);
+            int item = 0, st = 0;
+            const int more = list_rows_next(items, nitems, w, lane, walk_sh[w], item, st, y0, ly, together);
+            if (more < 0) break;
+            if (more == 0) continue;
+            strip = st;
+            load_seg(items[item].a, g);
             if (!emit) g.rho_out = nullptr;
-            local = u - items[it].unit_begin;
-            ns = items[it].nstrips;
-            bh = items[it].band;
-            __syncwarp();  // the previous unit's reads of gs are done
+            __syncwarp();  // the previous segment's reads of gs are done
             if (lane == 0) gs = g;
             __syncwarp();
+        } else {
+            const int64_t b = u / nstrips;
+            strip = u - b * nstrips;
+            y0 = (int)(b * band);
+            ly = (int)a.ny - y0 < (int)band ? (int)a.ny - y0 : (int)band;
         }
         // rows and columns fit 32 bits (sides <= 65535); plane offsets need 64
         const int nx = (int)g.nx, ny = (int)g.ny;
-        const int64_t b = local / ns, strip = local - b * ns;
-        const int y0 = (int)(b * bh);
-        const int ly = ny - y0 < (int)bh ? ny - y0 : (int)bh;
         const int xb = (int)(strip * WO) - HL;  // first window column (even)
         const int a0 = xb - (int)wrap_mod(xb, 4);  // first staged column
         const int o = xb - a0;                     // staged column of xb: 0 or 2
@@ -276,7 +294,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
             }
             {
                 const SegArgs cg = p_coll();
-                collide_pair<Q, S, RK>(cg, f0, f1, rho0, rho1);
+                collide(cg, f0, f1, rho0, rho1);
             }
 #pragma unroll
             for (int m = 1; m < K; ++m) {  // level m + 1 from level m (carried index m - 1)
@@ -335,7 +353,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
                         }
                 }
                 const SegArgs cg = p_coll();
-                collide_pair<Q, S, RK>(cg, f0, f1, rho0, rho1);
+                collide(cg, f0, f1, rho0, rho1);
             }
             if (j >= 2 * K) {  // level K of row y0 + j - 2K: window columns HL .. 63 - HL
                 const int x = xb + 2 * lane;
@@ -353,7 +371,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
                             for (int i = 0; i < Q; ++i)
                                 *reinterpret_cast<float2 *>(dp + (s * Q + i) * pl) = make_float2(f0[s][i], f1[s][i]);
                             if (rp) *reinterpret_cast<float2 *>(rp + s * pl + yx) = make_float2(rho0[s], rho1[s]);
-                            sum[s] += rho0[s] + rho1[s];
+                            if constexpr (!BATCH) sum[s] += rho0[s] + rho1[s];
                         }
                     } else if constexpr (ANY) {  // the last column of an odd nx
 #pragma unroll
@@ -361,19 +379,22 @@ __global__ void __launch_bounds__(NW * 32, MINB)
 #pragma unroll
                             for (int i = 0; i < Q; ++i) dp[(s * Q + i) * pl] = f0[s][i];
                             if (rp) rp[s * pl + yx] = rho0[s];
-                            sum[s] += rho0[s];
+                            if constexpr (!BATCH) sum[s] += rho0[s];
                         }
                     }
                 }
             }
-            __syncwarp();  // every lane has read slot j - 2 before iteration j + 1 stages into it
+            // every lane has read slot j - 2 before iteration j + 1 stages into it
+            if (BATCH && Q == 9 && together && (j & 3) == 0) __syncthreads();
+            else __syncwarp();
             sl = sl + 1 == NS ? 0 : sl + 1;
         }
 #pragma unroll
         for (int s = 0; s < S; ++s) acc[s] += (double)sum[s];
     }
     cp_async_wait<0>();
-    if (a.mass_out) block_mass_reduce<S, NW * 32>(acc, a.partials, a.counter, a.mass_out);
+    if constexpr (!BATCH)  // a list's masses come from its densities
+        if (a.mass_out) block_mass_reduce<S, NW * 32>(acc, a.partials, a.counter, a.mass_out);
 }
 
 template <int Q, int S, int K, int NW, int NS, int MINB, bool BATCH, bool PP = false, bool ANY = false, int RK = -1,

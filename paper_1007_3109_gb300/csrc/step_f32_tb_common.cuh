@@ -106,6 +106,46 @@ __device__ __forceinline__ void collide_pair(const Args &a, float (&f0)[S][Q], f
     }
 }
 
+// collide_pair with the two species' operands of a site packed in pairs
+// (FP32x2 instructions): a pull moves both species of a site alike, so the
+// pairs hold through the shifts and need no moves, unlike two columns'.
+template <int Q, int RK = -1, typename Args>
+__device__ __forceinline__ void collide_pair_species(const Args &a, float (&f0)[2][Q], float (&f1)[2][Q],
+                                                     float (&rho0)[2], float (&rho1)[2]) {
+    using L = Lattice<Q>;
+    float2 r0 = make_float2(f0[0][0], f0[1][0]), r1 = make_float2(f1[0][0], f1[1][0]);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+        r0 = rn_add2(r0, make_float2(f0[0][i], f0[1][i]));
+        r1 = rn_add2(r1, make_float2(f1[0][i], f1[1][i]));
+    }
+    rho0[0] = r0.x;
+    rho0[1] = r0.y;
+    rho1[0] = r1.x;
+    rho1[1] = r1.y;
+    float R0[2], R1[2];
+    reaction2_f32<2, RK>(a.rkind, (float)a.kappa, (float)a.F, (float)a.k, rho0, rho1, R0, R1);
+    const float2 om = make_float2((float)a.omega[0], (float)a.omega[1]);
+    const float2 c1 = make_float2(rn_sub(1.f, om.x), rn_sub(1.f, om.y));
+    const float2 t0 = rn_fma2(om, r0, make_float2(R0[0], R0[1]));
+    const float2 t1 = rn_fma2(om, r1, make_float2(R1[0], R1[1]));
+    float2 wt0[L::kClasses], wt1[L::kClasses];
+#pragma unroll
+    for (int c = 0; c < L::kClasses; ++c) {
+        wt0[c] = rn_mul2(pair2(L::template wc<float>(c)), t0);
+        wt1[c] = rn_mul2(pair2(L::template wc<float>(c)), t1);
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const float2 v0 = rn_fma2(c1, make_float2(f0[0][i], f0[1][i]), wt0[L::wclass(i)]);
+        const float2 v1 = rn_fma2(c1, make_float2(f1[0][i], f1[1][i]), wt1[L::wclass(i)]);
+        f0[0][i] = v0.x;
+        f0[1][i] = v0.y;
+        f1[0][i] = v1.x;
+        f1[1][i] = v1.y;
+    }
+}
+
 // The fields of one grid a multi-step segment needs, in registers (FP32 copies
 // of the relaxation rates and reaction constants: the values the one-step
 // kernels compute with).

@@ -31,7 +31,7 @@ int64_t plan_half_batch(DeepItem *items, int n) {
         using PS = HalfPairShape<K>;
         if (HalfPairKernel<Q, S, H, K, PS::NW, PS::NS, PS::MINB, true>::get(&full) != cudaSuccess) return -1;
         NW = PS::NW;
-        WO = PairGeom<K>::WO;
+        return plan_list_rows(items, n, PairGeom<K>::WO, NW);
     } else {
         using HS = HalfShape<K>;
         if (HalfDeepKernel<Q, S, H, K, HS::NW, HS::NS, HS::MINB, true>::get(&full) != cudaSuccess) return -1;
@@ -70,8 +70,8 @@ cudaError_t launch_half_pair_list(const DeepItem *items, int n, int64_t total_un
     unsigned full = 0;
     cudaError_t e = HK::get(&full);
     if (e != cudaSuccess) return e;
-    const int64_t nwarps = (int64_t)full * PS::NW;
-    const unsigned grid = total_units < nwarps ? (unsigned)((total_units + PS::NW - 1) / PS::NW) : full;
+    // total_units rows, shared out over the whole grid (at least one row per block)
+    const unsigned grid = total_units < (int64_t)full ? (unsigned)total_units : full;
     step_half_pair_kernel<Q, S, H, K, PS::NW, PS::NS, PS::MINB, true, RK>
         <<<grid, PS::NW * 32, HK::smem, st>>>(StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
     return cudaGetLastError();
