@@ -262,7 +262,9 @@ LB_RD_API const char *lb_rd_variant_name(int32_t precision, int32_t variant);
 /* The variants of one handle's configuration: configurations with more than
  * two species or a mass-action network run the general kernel, whose FP32
  * variants update 1, 2 or 4 consecutive sites per thread (nx a multiple of
- * that) and whose FP64 form has one variant.  Bitwise-equal results. */
+ * that) or run 2 or 3 steps per launch (gdeep<K>_, nx a multiple of 4, chosen
+ * by the autotuner or lb_rd_set_variant) and whose FP64 form has one variant.
+ * Bitwise-equal results. */
 LB_RD_API int lb_rd_handle_variant_count(const lb_rd_handle *h, int32_t *count);
 LB_RD_API const char *lb_rd_handle_variant_name(const lb_rd_handle *h, int32_t variant);
 LB_RD_API int lb_rd_autotune(lb_rd_handle *h, int32_t iters, int32_t *best, double *times_ms, int32_t max_times);

@@ -126,7 +126,8 @@ int handle_variant_count(const lb_rd_handle *h) {
 bool is_half(const lb_rd_handle *h) { return h->prec == LB_RD_FP32_BF16DEV || h->prec == LB_RD_FP32_FP16DEV; }
 
 int variant_steps(const lb_rd_handle *h, int v) {
-    if (h->general || h->inplace || v < 0) return 1;
+    if (h->inplace || v < 0) return 1;
+    if (h->general) return h->prec == LB_RD_FP64 ? 1 : lbrd::kGeneralVariants[v].steps;
     if (h->prec == LB_RD_FP32) return lbrd::kF32Variants[v].steps;
     return is_half(h) ? lbrd::kHalfVariantSteps[v] : 1;
 }
@@ -139,9 +140,10 @@ bool variant_fits(const lb_rd_handle *h, int v) {
 }
 
 // A variant of a depth-K kernel (it can write the densities of its last level):
-// the FP32 ones and the 16-bit deviation ones of two or more steps.
+// the FP32 ones and the general and 16-bit deviation ones of two or more steps.
 bool is_deep(const lb_rd_handle *h, int v) {
-    if (h->general || h->inplace || v < 0) return false;
+    if (h->inplace || v < 0) return false;
+    if (h->general) return variant_steps(h, v) >= 2;
     if (h->prec == LB_RD_FP32) return lbrd::kF32Variants[v].cache == 4;
     return is_half(h) && lbrd::kHalfVariantSteps[v] >= 2;
 }

@@ -62,10 +62,12 @@ struct StepShape {
 struct GeneralVariant {
     const char *name;
     int sites;  // consecutive sites per thread; the variant needs nx % sites == 0
+    int steps;  // time steps per launch; 2 or more: step_general_deep.cu, writes rho of its last step
 };
 extern const GeneralVariant kGeneralVariants[];
 extern const int kGeneralVariantCount;  // FP32; FP64 has variant 0 only
 cudaError_t launch_step_general(int prec, int Q, int S, const StepArgs &a, cudaStream_t st, int variant);
+cudaError_t launch_step_general_deep(int v, int Q, int S, const StepArgs &a, cudaStream_t st);
 cudaError_t launch_init_general(int prec, int Q, int S, const InitArgs &a, cudaStream_t st);
 
 // In-place (AA) step: phase 0 for t even (natural in, pushed-and-swapped

@@ -146,7 +146,7 @@ cudaError_t aa_vec(int Q, int S, int phase, const StepArgs &a, cudaStream_t st) 
 
 }  // namespace
 
-const GeneralVariant kAAVariants[] = {{"aa_1site", 1}, {"aa_2site", 2}, {"aa_4site", 4}, {"aa_4site_minb3", 4}};
+const GeneralVariant kAAVariants[] = {{"aa_1site", 1, 1}, {"aa_2site", 2, 1}, {"aa_4site", 4, 1}, {"aa_4site_minb3", 4, 1}};
 const int kAAVariantCount = sizeof(kAAVariants) / sizeof(kAAVariants[0]);
 
 cudaError_t launch_step_aa(int prec, int Q, int S, int phase, const StepArgs &a, cudaStream_t st, int variant) {
