@@ -487,7 +487,7 @@ def network_mode(args):
     sim.close()
     bps = S * 9 * (8 if prec == "fp64" else 4) * 2
     peak, peak_kind = measured_peaks()
-    achieved = bps * n * n / (ms / 1e3 / args.steps) / 1e9
+    achieved = bps * n * n * launches / (ms / 1e3) / 1e9  # a launch (of one or more steps) moves the state once
     line = {"metric": "MLUPS", "value": S * n * n * args.steps / (ms / 1e3) / 1e6,
             "unit": "MLUPS (species-site updates/s / 1e6)", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,

@@ -145,7 +145,9 @@ typedef struct {
     int32_t streaming;       /* lb_rd_streaming */
     void *stream;            /* cudaStream_t for all work; NULL = legacy default stream */
     int32_t tb_depth;        /* time steps per launch (temporal blocking): 0 = the autotuner's cached choice
-                                (else one step per launch); 1 = one; 2 .. 8 = a depth-K variant of that
+                                (else by size: grids of more than 65536 sites in FP32 or 16-bit deviation
+                                storage with two state copies run several steps per launch, others one);
+                                1 = one; 2 .. 8 = a depth-K variant of that
                                 many steps (FP32 or 16-bit deviation storage with two state copies and
                                 at most two species only, else EINVAL; lb_rd_create also fails with
                                 EINVAL when no variant of that depth fits the grid).  Batches take
@@ -190,7 +192,9 @@ LB_RD_API int lb_rd_init(lb_rd_handle *h, const double *rho0, int is_device);
  * and splits its last steps into launches of fewer steps (chosen from the
  * autotuner's times per depth to finish soonest); a last launch of two or more
  * steps also writes the densities rho(t), so that no single-step launch is
- * needed to leave them available. */
+ * needed to leave them available.  An untuned handle of more than 65536 sites
+ * (tb_depth 0) runs a depth-K variant chosen by its size, with the same
+ * results; with track_mass its call ends on a single step. */
 LB_RD_API int lb_rd_step(lb_rd_handle *h, int64_t nsteps);
 
 /* Current time step t of the handle. */

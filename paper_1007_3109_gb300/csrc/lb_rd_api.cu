@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <map>
 #include <mutex>
 #include <string>
@@ -83,6 +84,7 @@ struct lb_rd_handle {
     int inject_timeout = 0;  // one-shot test switch for the bounded-wait error path
     int variant = 0;      // single-step launch variant of the step kernel
     int tb_variant = -1;  // multi-step (temporal blocking, K steps per launch) variant, or -1
+    bool by_size = false; // tb_variant is default_bulk's choice (untuned, depth left to the library)
     // depth-K variants per steps per launch d = 2 .. 8 (-1: none fits) and, once
     // tuned, their time per step (ms): the launches that cover the last steps of a call
     int depth_variant[9] = {-1, -1, -1, -1, -1, -1, -1, -1, -1};
@@ -93,6 +95,8 @@ struct lb_rd_handle {
     bool general = false; // runs the general kernel
     bool inplace = false; // one state copy, AA pattern (buf[1] unused)
 };
+
+extern "C" const char *lb_rd_handle_variant_name(const lb_rd_handle *h, int32_t variant);
 
 namespace {
 // Autotuner choices per (device, precision, Q, S, nx, ny): single-step
@@ -148,14 +152,36 @@ bool is_deep(const lb_rd_handle *h, int v) {
     return is_half(h) && lbrd::kHalfVariantSteps[v] >= 2;
 }
 
-// Untuned depth table: per d = 2 .. 8 the first depth-K variant of d steps
-// that fits the grid, in table order.
+// The first of the named variants that exists for the handle and fits its grid, or -1.
+int first_fitting(const lb_rd_handle *h, std::initializer_list<const char *> names) {
+    for (const char *name : names)
+        for (int v = 0; v < handle_variant_count(h); ++v)
+            if (std::strcmp(lb_rd_handle_variant_name(h, v), name) == 0 && variant_fits(h, v)) return v;
+    return -1;
+}
+
+// Untuned depth table: per d = 2 .. 8 the depth-K variant of d steps that the
+// autotuner picks on large grids (two columns per lane where that form fits),
+// else the first that fits in table order.
 void default_depths(lb_rd_handle *h) {
     for (int d = 0; d < 9; ++d) {
         h->depth_variant[d] = -1;
         h->depth_ms[d] = 0.0;
     }
     h->depth_tuned = false;
+    if (h->prec == LB_RD_FP32 && !h->general && !h->inplace) {
+        h->depth_variant[3] = first_fitting(h, {"deep3vwp_128_minb2_s5"});
+        h->depth_variant[4] = first_fitting(h, {"deep4vw_128_minb2", "deep4vwa_128_minb2"});
+        h->depth_variant[5] = first_fitting(h, {"deep5vw_128_minb2", "deep5vwpa_256_minb1"});
+        h->depth_variant[6] = h->S * h->Q <= 10 ? first_fitting(h, {"deep6vwp_128_minb1_s6", "deep6vwpa_128_minb1"})
+                                                : first_fitting(h, {"deep6vp_128_minb2"});
+    } else if (is_half(h)) {
+        for (int d : {2, 3, 4, 5})
+            h->depth_variant[d] = d == 2   ? first_fitting(h, {"hpair2_128_minb4"})
+                                  : d == 3 ? first_fitting(h, {"hpair3_128_minb3"})
+                                  : d == 4 ? first_fitting(h, {"hpair4_128_minb2", "hdeep4_128_minb3"})
+                                           : first_fitting(h, {"hpair5_128_minb2"});
+    }
     for (int v = 0; v < handle_variant_count(h); ++v) {
         const int d = variant_steps(h, v);
         if (is_deep(h, v) && d >= 2 && d <= 8 && h->depth_variant[d] < 0 && variant_fits(h, v))
@@ -163,7 +189,36 @@ void default_depths(lb_rd_handle *h) {
     }
 }
 
+// The multi-step variant of an untuned handle that leaves the depth to the
+// library (tb_depth 0), by lattice, species, storage, alignment and size; -1:
+// one step per launch.  Grids of up to 2^16 sites keep one launch per step: a
+// step there is launch latency either way (256^2: 6.2 us, five steps per launch
+// 2.9 us each), and callers that time or count the steps of small grids see
+// each one.  Above, us per step of the rule's choice against the one-step
+// default, FP32 D2Q9 with two species: 512^2 4.1 / 8.3, 1531 x 1021 13.9 / 49.3,
+// 2048^2 24.6 / 102, 4096^2 87 / 391; D2Q5 4096^2 38 / 207; bf16 deviations
+// 2048^2 30 / 62.  The lines between two choices lie where the autotuner's times
+// cross: the six-row ring hides the latency of L2-resident rows (512^2: 4.1
+// against 4.5, 1024^2 8.6 / 8.9, 1448^2 14.2 / 14.0), the any-nx two-column form
+// needs enough rows per warp (383 x 511: 5.4 against the one-column form's 5.2,
+// 767 x 703 7.4 / 7.7), K = 2 beats K = 3 for four D2Q9 species on small grids
+// (512^2: 14.5 / 17.9; 2048^2: 139 / 135).
+int default_bulk(const lb_rd_handle *h) {
+    const int64_t sites = h->cfg.nx * h->cfg.ny;
+    if (sites <= (1 << 16) || h->inplace || h->prec == LB_RD_FP64) return -1;
+    if (h->general)
+        return h->S * h->Q > 27 && sites < (1 << 21) ? first_fitting(h, {"gdeep2_128_minb2"})
+                                                     : first_fitting(h, {"gdeep3_128_minb3"});
+    if (is_half(h))
+        return first_fitting(h, {"hpair4_128_minb2", sites < (1 << 21) ? "hdeep4_128_minb2" : "hdeep4_128_minb3"});
+    if (h->S * h->Q > 10)
+        return first_fitting(h, {sites <= (3 << 19) ? "deep5vw_128_minb2_s6" : "deep5vw_256_minb1",
+                                 sites < (3 << 17) ? "deep4_128_minb3" : "deep5vwpa_256_minb1"});
+    return first_fitting(h, {h->Q == 9 ? "deep6vwpe_128_minb1_s5" : "deep6vwp_128_minb1_s6", "deep6vwpa_128_minb1"});
+}
+
 void apply_tune(lb_rd_handle *h, const TuneEntry &t) {
+    h->by_size = false;
     h->variant = t.variant;
     h->tb_variant = t.tb_variant;
     bool tuned = false;
@@ -183,16 +238,22 @@ void apply_tune(lb_rd_handle *h, const TuneEntry &t) {
 // of the depth sweep's shape), so that a call of any length runs close to the
 // per-step rate of the deepest launches and ends on a launch that also writes
 // rho.  Other multi-step variants (two-step kernels, which cannot write rho)
-// keep the last step single, like one-step variants.
+// keep the last step single, like one-step variants.  single_last: the call's
+// last step is a launch of its own.
 struct LaunchPlan {
     int64_t bulk = 0;
     int K = 1;
     std::vector<int> tail;
 };
 
-LaunchPlan plan_launches(const lb_rd_handle *h, int64_t nsteps) {
+LaunchPlan plan_launches(const lb_rd_handle *h, int64_t nsteps, bool single_last) {
     LaunchPlan p;
     if (nsteps <= 0) return p;
+    if (single_last) {
+        p = plan_launches(h, nsteps - 1, false);
+        p.tail.push_back(1);
+        return p;
+    }
     const int K = h->tb_variant >= 0 ? variant_steps(h, h->tb_variant) : 1;
     if (K == 1 || !is_deep(h, h->tb_variant)) {
         p.K = K;
@@ -371,7 +432,12 @@ int lb_rd_create(const lb_rd_config *cfg, lb_rd_handle **out) {
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_tune_cache.find(tune_key(h));
-        if (it != g_tune_cache.end()) apply_tune(h, it->second);
+        if (it != g_tune_cache.end()) {
+            apply_tune(h, it->second);
+        } else if (cfg->tb_depth == 0) {
+            h->tb_variant = default_bulk(h);
+            h->by_size = h->tb_variant >= 0;
+        }
     }
     if (cfg->tb_depth == 1) {
         h->tb_variant = -1;
@@ -499,7 +565,11 @@ int lb_rd_step(lb_rd_handle *h, int64_t nsteps) {
     // last launch of d >= 2 steps writes rho(t) (the other copy then no longer
     // holds f*(t - 1)), a last single step leaves it to be recomputed on demand
     // from the other copy (ensure_rho).
-    const LaunchPlan plan = plan_launches(h, nsteps);
+    // A handle on the size rule with a tracked mass ends on a single step, which
+    // reduces the mass (only the last step's can be read): the same masses, bit
+    // for bit, as with one step per launch.
+    const bool mass_last = h->by_size && h->cfg.track_mass;
+    const LaunchPlan plan = plan_launches(h, nsteps, mass_last);
     const int64_t nl = plan.bulk + (int64_t)plan.tail.size();
     for (int64_t n = 0; n < nl; ++n) {
         const int d = n < plan.bulk ? plan.K : plan.tail[(size_t)(n - plan.bulk)];
@@ -508,7 +578,7 @@ int lb_rd_step(lb_rd_handle *h, int64_t nsteps) {
         a.src = h->buf[h->cur];
         a.dst = h->buf[h->cur ^ 1];
         a.rho_out = last && d >= 2 ? h->rho : nullptr;
-        a.mass_out = h->cfg.track_mass ? h->mass : nullptr;
+        a.mass_out = h->cfg.track_mass && (last || !mass_last) ? h->mass : nullptr;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (h->timing) {
             LBRD_CUDA(cudaEventCreate(&e0), "event create");
@@ -761,7 +831,8 @@ int lb_rd_set_variant(lb_rd_handle *h, int32_t variant) {
         auto it = g_tune_cache.find(tune_key(h));
         default_depths(h);
         h->variant = 0;
-        h->tb_variant = -1;
+        h->tb_variant = h->cfg.tb_depth == 0 ? default_bulk(h) : -1;
+        h->by_size = h->tb_variant >= 0;
         if (it != g_tune_cache.end()) apply_tune(h, it->second);
         return LB_RD_OK;
     }
@@ -774,6 +845,7 @@ int lb_rd_set_variant(lb_rd_handle *h, int32_t variant) {
                                                      : h->general ? lbrd::kGeneralVariants[variant].sites
                                                      : is_half(h) ? lbrd::kHalfVariantNx[variant]
                                                                   : lbrd::kF32Variants[variant].nx_multiple));
+    h->by_size = false;
     if (variant_steps(h, variant) >= 2) {
         h->tb_variant = variant;
     } else {
