@@ -177,7 +177,7 @@ cudaError_t launch_batch_tb2(const TbwItem *items, int n, int64_t total_units, i
 struct DeepItem {
     StepArgs a;
     int64_t unit_begin, nstrips, band;
-    int64_t run_strips, next;  // two-column kernels: the list's rows (list_rows.cuh)
+    int64_t run_strips, next, height;  // two-column kernels: the list's rows (list_rows.cuh)
     int gs, lockstep;
 };
 // The same over 16-bit deviation storage (K = 2 .. 5; half_kind 0 bf16, 1 fp16;

@@ -88,7 +88,7 @@ int64_t plan_batch(DeepItem *items, int n) {
         ge = BatchShape<Q, S, K, V16>::get(&full);
     }
     if (ge != cudaSuccess) return -1;
-    if constexpr (pair) return plan_list_rows(items, n, WO, NW);
+    if constexpr (pair) return plan_list_rows(items, n, K, WO, NW, full);
     for (int i = 0; i < n; ++i) items[i].nstrips = (items[i].a.nx + WO - 1) / WO;
     const int64_t h = choose_band_height(K, items, n, (int64_t)full * NW);
     int64_t units = 0;

@@ -144,9 +144,8 @@ __global__ void __launch_bounds__(NW * 32, MINB)
             return g;
         }
     };
-    // lists of two-species D2Q9 grids: the species of a site packed (1024 x 256^2 at K = 5 runs at
-    // 98 against 99.4 us per step and quarter, one 512^2 grid at 4.8 against 5.5; D2Q5 and single grids
-    // gain nothing)
+    // lists of two-species D2Q9 grids: the species of a site packed (256 x 256^2 at K = 5: 98.0 against
+    // 99.4 us per step, 256 x 255^2 137 / 145, 9 x 512^2 16.7 / 17.6; D2Q5 and single grids gain nothing)
     auto collide = [](const SegArgs &cg, float(&f0)[S][Q], float(&f1)[S][Q], float(&rho0)[S], float(&rho1)[S]) {
         if constexpr (BATCH && Q == 9 && S == 2) collide_pair_species<Q, RK>(cg, f0, f1, rho0, rho1);
         else collide_pair<Q, S, RK>(cg, f0, f1, rho0, rho1);

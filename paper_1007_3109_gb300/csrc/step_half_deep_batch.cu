@@ -31,7 +31,7 @@ int64_t plan_half_batch(DeepItem *items, int n) {
         using PS = HalfPairShape<K>;
         if (HalfPairKernel<Q, S, H, K, PS::NW, PS::NS, PS::MINB, true>::get(&full) != cudaSuccess) return -1;
         NW = PS::NW;
-        return plan_list_rows(items, n, PairGeom<K>::WO, NW);
+        return plan_list_rows(items, n, K, PairGeom<K>::WO, NW, full);
     } else {
         using HS = HalfShape<K>;
         if (HalfDeepKernel<Q, S, H, K, HS::NW, HS::NS, HS::MINB, true>::get(&full) != cudaSuccess) return -1;
