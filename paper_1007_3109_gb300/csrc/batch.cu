@@ -625,25 +625,21 @@ int lb_rd_batch_moments(lb_rd_batch *b, int32_t idx, double *rho_out, double *ma
     const lb_rd_config &c = b->cfgs[idx];
     const void *rho = b->rho + b->rho_off[idx];
     const size_t n = (size_t)b->S * c.ny * c.nx;
-    if (rho_out) {
+    if (rho_out || mass_out) {  // one pass over the density cache for both
         double *dst = rho_out;
-        if (!is_device) {
+        if (rho_out && !is_device) {
             int rc = batch_stage(b, n);
             if (rc) return rc;
             dst = b->stage;
         }
-        cudaError_t e = lbrd::launch_rho_export(b->prec, b->S, rho, c.nx, c.ny, b->pitch[idx], dst, b->stream);
-        if (!e && !is_device) e = cudaMemcpyAsync(rho_out, b->stage, n * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
-        if (e) return cuda_err(e, "batch rho export");
-        b->launches++;
-    }
-    if (mass_out) {
-        cudaError_t e = lbrd::launch_mass(b->prec, b->S, rho, c.nx, c.ny, b->pitch[idx], b->partials, b->counter,
-                                          b->mass, b->stream);
-        if (!e)
-            e = cudaMemcpyAsync(mass_out, b->mass, b->S * sizeof(double),
-                                is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, b->stream);
-        if (e) return cuda_err(e, "batch mass");
+        double *mass = !mass_out ? nullptr : (is_device ? mass_out : b->mass);
+        cudaError_t e = lbrd::launch_readout(b->prec, b->S, rho, c.nx, c.ny, b->pitch[idx], dst, b->partials,
+                                             b->counter, mass, b->stream);
+        if (!e && rho_out && !is_device)
+            e = cudaMemcpyAsync(rho_out, b->stage, n * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
+        if (!e && mass_out && !is_device)
+            e = cudaMemcpyAsync(mass_out, b->mass, b->S * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
+        if (e) return cuda_err(e, "batch readout");
         b->launches++;
     }
     cudaError_t e = cudaStreamSynchronize(b->stream);

@@ -620,32 +620,27 @@ int lb_rd_moments(lb_rd_handle *h, double *rho_out, double *mass_out, int is_dev
         int rc = ensure_rho(h);
         if (rc) return rc;
     }
-    if (rho_out) {
+    const bool sum = mass_out && !h->mass_fresh;
+    if (rho_out || sum) {  // one pass over the density cache for both
         double *dst = rho_out;
-        if (!is_device) {
+        if (rho_out && !is_device) {
             int rc = ensure_stage(h, n);
             if (rc) return rc;
             dst = h->stage;
         }
-        cudaError_t e = lbrd::launch_rho_export(h->prec, h->S, h->rho, nx, ny, h->pitch, dst, h->stream);
-        if (e) return cuda_fail(e, "rho export kernel");
+        cudaError_t e = lbrd::launch_readout(h->prec, h->S, h->rho, nx, ny, h->pitch, dst, h->partials, h->counter,
+                                             sum ? h->mass : nullptr, h->stream);
+        if (e) return cuda_fail(e, "readout kernel");
         h->launches++;
-        if (!is_device)
+        if (sum) h->mass_fresh = true;
+        if (rho_out && !is_device)
             LBRD_CUDA(cudaMemcpyAsync(rho_out, h->stage, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
                       "rho download");
     }
-    if (mass_out) {
-        if (!h->mass_fresh) {
-            cudaError_t e = lbrd::launch_mass(h->prec, h->S, h->rho, nx, ny, h->pitch, h->partials, h->counter,
-                                              h->mass, h->stream);
-            if (e) return cuda_fail(e, "mass kernel");
-            h->launches++;
-            h->mass_fresh = true;
-        }
+    if (mass_out)
         LBRD_CUDA(cudaMemcpyAsync(mass_out, h->mass, h->S * sizeof(double),
                                   is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream),
                   "mass download");
-    }
     int status = 0;
     LBRD_CUDA(cudaMemcpyAsync(&status, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "status read");
     LBRD_CUDA(cudaStreamSynchronize(h->stream), "moments sync");

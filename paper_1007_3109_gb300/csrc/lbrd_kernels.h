@@ -136,12 +136,11 @@ cudaError_t launch_export(int prec, int Q, int S, const void *state, int64_t nx,
                           double *out, cudaStream_t st);
 
 // rho cache ([s][y][pitch] in double (prec 0) or float) to packed FP64
-// [s][y][x], and its global FP64 sum per species.
-cudaError_t launch_rho_export(int prec, int S, const void *rho, int64_t nx, int64_t ny, int64_t pitch,
-                              double *out, cudaStream_t st);
+// [s][y][x] (out, or null) and its global FP64 sum per species (mass, or null;
+// partials holds mass_partials_needed(nx, ny) * S doubles).
 size_t mass_partials_needed(int64_t nx, int64_t ny);
-cudaError_t launch_mass(int prec, int S, const void *rho, int64_t nx, int64_t ny, int64_t pitch,
-                        double *partials, unsigned int *counter, double *mass, cudaStream_t st);
+cudaError_t launch_readout(int prec, int S, const void *rho, int64_t nx, int64_t ny, int64_t pitch, double *out,
+                           double *partials, unsigned int *counter, double *mass, cudaStream_t st);
 
 // Batched step: one persistent launch over the combined (instance x tile)
 // work list.  Tiles are 256 x 2 sites (64 x 2 threads, 4 sites each); the

@@ -179,12 +179,10 @@ int collect_request(lb_rd_server *s, Request *r) {
         e = cudaMallocAsync((void **)&s->partials, parts * sizeof(double), s->stream);
         if (!e) s->partials_cap = parts;
     }
-    if (!e) e = lbrd::launch_rho_export(prec, c.nspecies, r->rho, c.nx, c.ny, r->pitch, stage, s->stream);
+    if (!e) e = lbrd::launch_readout(prec, c.nspecies, r->rho, c.nx, c.ny, r->pitch, stage, s->partials, s->counter,
+                                     s->d_mass, s->stream);
     r->rho_out.resize(n);
     if (!e) e = cudaMemcpyAsync(r->rho_out.data(), stage, n * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
-    if (!e)
-        e = lbrd::launch_mass(prec, c.nspecies, r->rho, c.nx, c.ny, r->pitch, s->partials, s->counter, s->d_mass,
-                              s->stream);
     if (!e) e = cudaMemcpyAsync(r->mass, s->d_mass, c.nspecies * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
     if (stage) cudaFreeAsync(stage, s->stream);
     if (!e) e = cudaStreamSynchronize(s->stream);
