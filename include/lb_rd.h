@@ -429,7 +429,7 @@ LB_RD_API int lb_rd_server_stats(const lb_rd_server *srv, int64_t *launches, int
  * Scratch: the reduction's per-block partial sums and its arrival counter
  * live in a static device array of 65536 doubles plus 256 bytes (512 KiB),
  * held by every GPU that loads the library until the process exits.  One
- * block runs per tile (256 x 2 sites in FP32 and 16-bit storage, 32 x 4
+ * block runs per tile at most (256 x 2 sites in FP32 and 16-bit storage, 32 x 4
  * sites in FP64), and the grid's tiles times S may not exceed 65536: for two
  * species that is up to 16.7 million FP32 sites (4096 x 4096) or 4.2 million
  * FP64 sites (2048 x 2048).  Larger grids return LB_RD_EINVAL with the

@@ -25,13 +25,12 @@ int report_error(int code, const std::string &msg);
 namespace {
 
 constexpr int kBX = 64, kBY = 2, kNT = kBX * kBY;  // the tile shape of both tile bodies
-static_assert(half::kBX == kBX && half::kBY == kBY, "tile shapes must agree");
+static_assert(half::kBX == kBX && half::kBY == kBY && f64::kNT == kNT, "tile shapes must agree");
 
 // MODE 0: FP32 storage, 1: bf16 deviations, 2: fp16 deviations, 3: FP64,
 // 4: FP32 where some instances keep one copy updated in place (the AA tile
 // body of step_aa_kernel.cuh; BatchItem::aa selects the body per instance).
-// An FP64 tile covers the same 256 x 2 sites; a thread updates the sites
-// x = x_tile + threadIdx.x + 64 j, j < 4 (coalesced), one at a time.
+// An FP64 tile is 128 consecutive sites (step_f64_kernel.cuh), the others 256 x 2.
 template <int Q, int S, int MODE>
 __global__ void __launch_bounds__(kNT, 4) batch_kernel(const BatchItem *__restrict__ items, int nitems,
                                                        int64_t total_tiles) {
@@ -42,20 +41,23 @@ __global__ void __launch_bounds__(kNT, 4) batch_kernel(const BatchItem *__restri
     for (int s = 0; s < S; ++s) acc[s] = 0.0;
     int it = 0;
     for (int64_t t = blockIdx.x; t < total_tiles; t += gridDim.x) {
-        while (it + 1 < nitems && items[it + 1].tile_begin <= t) ++it;
-        const BatchItem &b = items[it];
-        const int64_t local = t - b.tile_begin;
-        const int64_t ty = local / b.tiles_x, tx = local - ty * b.tiles_x;
-        const int64_t y = ty * kBY + threadIdx.y;
-        if constexpr (MODE == 3) {
-            if (y < b.a.ny) {
-#pragma unroll 1
-                for (int j = 0; j < 4; ++j) {
-                    const int64_t x = tx * kBX * 4 + threadIdx.x + j * kBX;
-                    if (x < b.a.nx) f64::site_f64<Q, S>(b.a, x, y, acc);
-                }
+        if constexpr (MODE == 3) {  // a block of its own per tile: bisection instead of a scan from the first item
+            int hi = nitems;
+            while (hi - it > 1) {
+                const int mid = (it + hi) / 2;
+                if (items[mid].tile_begin <= t) it = mid;
+                else hi = mid;
             }
         } else {
+            while (it + 1 < nitems && items[it + 1].tile_begin <= t) ++it;
+        }
+        const BatchItem &b = items[it];
+        const int64_t local = t - b.tile_begin;
+        if constexpr (MODE == 3) {
+            f64::tile_f64<Q, S>(b.a, local, threadIdx.x + threadIdx.y * kBX, acc);
+        } else {
+            const int64_t ty = local / b.tiles_x, tx = local - ty * b.tiles_x;
+            const int64_t y = ty * kBY + threadIdx.y;
             const int64_t x0 = (tx * kBX + threadIdx.x) * 4;
             if constexpr (MODE == 0) {
                 f32::tile_f32<Q, S, 0>(b.a, x0, y, lane, acc);
@@ -84,7 +86,8 @@ __global__ void __launch_bounds__(kNT, 4) batch_kernel(const BatchItem *__restri
 template <int Q, int S, int MODE>
 cudaError_t launch_batch(const BatchItem *items, int n, int64_t total, cudaStream_t st) {
     auto kern = batch_kernel<Q, S, MODE>;
-    const unsigned grid = persistent_blocks(kern, kNT, total);
+    // FP64: one block per tile, as for a single grid (no mass is reduced here)
+    const unsigned grid = MODE == 3 && total < (1 << 30) ? (unsigned)total : persistent_blocks(kern, kNT, total);
     kern<<<grid, dim3(kBX, kBY), 0, st>>>(items, n, total);
     return cudaGetLastError();
 }
@@ -121,7 +124,9 @@ cudaError_t launch_batch_init(int mode, int Q, int S, const InitArgs &a, cudaStr
 
 int64_t batch_tiles_x(int64_t nx) { return ((nx + 3) / 4 + kBX - 1) / kBX; }
 
-int64_t batch_tiles(int64_t nx, int64_t ny) { return batch_tiles_x(nx) * ((ny + kBY - 1) / kBY); }
+int64_t batch_tiles(int mode, int64_t nx, int64_t ny) {
+    return mode == 3 ? f64::tiles(nx, ny) : batch_tiles_x(nx) * ((ny + kBY - 1) / kBY);
+}
 
 cudaError_t launch_batch_step(int mode, int Q, int S, const BatchItem *items, int n, int64_t total_tiles,
                              cudaStream_t st) {
@@ -341,7 +346,7 @@ int lb_rd_batch_create(const lb_rd_config *cfgs, int32_t n, lb_rd_batch **out) {
         it.a.k = c.reaction.k;
         it.tiles_x = lbrd::batch_tiles_x(c.nx);
         it.tile_begin = b->total_tiles;
-        b->total_tiles += lbrd::batch_tiles(c.nx, c.ny);
+        b->total_tiles += lbrd::batch_tiles(b->mode, c.nx, c.ny);
     }
     cudaError_t e = cudaSuccess;
     if (!e) e = cudaMalloc(&b->buf[0], b->state_total);

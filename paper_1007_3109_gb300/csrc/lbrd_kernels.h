@@ -143,8 +143,8 @@ cudaError_t launch_readout(int prec, int S, const void *rho, int64_t nx, int64_t
                            double *partials, unsigned int *counter, double *mass, cudaStream_t st);
 
 // Batched step: one persistent launch over the combined (instance x tile)
-// work list.  Tiles are 256 x 2 sites (64 x 2 threads, 4 sites each); the
-// instance of global tile t is the last item with tile_begin <= t.
+// work list.  Tiles are 256 x 2 sites (64 x 2 threads, 4 sites each; FP64: 128
+// consecutive sites); the instance of global tile t is the last item with tile_begin <= t.
 struct BatchItem {
     StepArgs a;          // per-instance grid, parameters and buffers
     int64_t tiles_x;     // tiles per row of tiles, ceil(ceil(nx / 4) / 64)
@@ -212,7 +212,7 @@ inline int list_reaction_kind(const DeepItem *items, int n) {
     return items[0].a.rkind;
 }
 int64_t batch_tiles_x(int64_t nx);
-int64_t batch_tiles(int64_t nx, int64_t ny);
+int64_t batch_tiles(int mode, int64_t nx, int64_t ny);
 // mode: 0 FP32 storage, 1 bf16 deviations, 2 fp16 deviations, 3 FP64,
 // 4 FP32 with in-place instances (BatchItem::aa).
 int batch_mode(int precision);

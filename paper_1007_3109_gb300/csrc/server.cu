@@ -342,7 +342,7 @@ void run_tick(lb_rd_server *s) {
         it.a.k = c.reaction.k;
         it.tiles_x = lbrd::batch_tiles_x(c.nx);
         it.tile_begin = total;
-        total += lbrd::batch_tiles(c.nx, c.ny);
+        total += lbrd::batch_tiles(s->mode, c.nx, c.ny);
         for (int set = 0; set < 3; ++set) {
             const int par = set < 2 ? (r->cur + set) & 1 : (int)((r->cur + L - 1) & 1);
             lbrd::BatchItem v = it;

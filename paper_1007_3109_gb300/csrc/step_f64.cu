@@ -1,6 +1,8 @@
-// FP64 step kernels: a persistent grid over 32 x 4 site tiles running the
-// per-site update of step_f64_kernel.cuh.  GB300's FP64 rate, not HBM, bounds
-// them.
+// FP64 step kernels: one block per tile of 128 consecutive sites running the
+// per-site update of step_f64_kernel.cuh (the hardware's block scheduler then
+// evens out the SMs and overlaps one block's loads with the others' arithmetic);
+// a persistent grid over the tiles where the mass is reduced, whose blocks leave
+// one partial sum each.  GB300's FP64 rate, not HBM, bounds them.
 #include "lbrd_kernels.h"
 #include "step_f64_kernel.cuh"
 
@@ -8,21 +10,15 @@ namespace lbrd {
 
 namespace {
 
-constexpr int kBX = 32, kBY = 4, kNT = kBX * kBY;
+constexpr int kBX = 32, kBY = 4, kNT = kBX * kBY;  // the initialisation's tile
+static_assert(kNT == f64::kNT, "one block size");
 
 template <int Q, int S>
-__global__ void __launch_bounds__(kNT) step_f64_kernel(StepArgs a, int64_t tiles_x, int64_t ntiles) {
+__global__ void __launch_bounds__(kNT) step_f64_kernel(StepArgs a, int64_t ntiles) {
     double acc[S];
 #pragma unroll
     for (int s = 0; s < S; ++s) acc[s] = 0.0;
-
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t ty = tile / tiles_x, tx = tile - ty * tiles_x;
-        const int64_t x = tx * kBX + threadIdx.x;
-        const int64_t y = ty * kBY + threadIdx.y;
-        if (x >= a.nx || y >= a.ny) continue;
-        f64::site_f64<Q, S>(a, x, y, acc);
-    }
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) f64::tile_f64<Q, S>(a, tile, threadIdx.x, acc);
     if (a.mass_out) block_mass_reduce<S, kNT>(acc, a.partials, a.counter, a.mass_out);
 }
 
@@ -65,16 +61,15 @@ dim3 grid_for(int64_t nx, int64_t ny) {
 
 template <int Q, int S>
 cudaError_t launch_tiles(const StepArgs &a, cudaStream_t st) {
-    const int64_t tiles_x = (a.nx + kBX - 1) / kBX;
-    const int64_t ntiles = tiles_x * ((a.ny + kBY - 1) / kBY);
-    const unsigned grid = persistent_blocks(step_f64_kernel<Q, S>, kNT, ntiles);
-    step_f64_kernel<Q, S><<<grid, dim3(kBX, kBY), 0, st>>>(a, tiles_x, ntiles);
+    const int64_t ntiles = f64::tiles(a.nx, a.ny);
+    const unsigned grid = a.mass_out ? persistent_blocks(step_f64_kernel<Q, S>, kNT, ntiles) : (unsigned)ntiles;
+    step_f64_kernel<Q, S><<<grid, kNT, 0, st>>>(a, ntiles);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-StepShape step_shape_f64(int64_t, int64_t) { return {dim3(max_persistent_blocks()), dim3(kBX, kBY)}; }
+StepShape step_shape_f64(int64_t, int64_t) { return {dim3(max_persistent_blocks()), dim3(kNT)}; }
 
 cudaError_t launch_step_f64(int Q, int S, const StepArgs &a, cudaStream_t st) {
     if (Q == 9 && S == 1) return launch_tiles<9, 1>(a, st);
@@ -94,15 +89,15 @@ cudaError_t launch_init_f64(int Q, int S, const InitArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// One block per tile instead of the persistent grid (allocation-free entry).
+// One block per tile also with the mass (allocation-free entry).  The entry point's
+// limit counts 32 x 4 tiles, of which there are never fewer than blocks.
 int64_t step_tiles_f64(int64_t nx, int64_t ny) { return ((nx + kBX - 1) / kBX) * ((ny + kBY - 1) / kBY); }
 
 namespace {
 template <int Q, int S>
 cudaError_t launch_per_tile(const StepArgs &a, cudaStream_t st) {
-    const int64_t tiles_x = (a.nx + kBX - 1) / kBX;
-    const int64_t ntiles = tiles_x * ((a.ny + kBY - 1) / kBY);
-    step_f64_kernel<Q, S><<<(unsigned)ntiles, dim3(kBX, kBY), 0, st>>>(a, tiles_x, ntiles);
+    const int64_t ntiles = f64::tiles(a.nx, a.ny);
+    step_f64_kernel<Q, S><<<(unsigned)ntiles, kNT, 0, st>>>(a, ntiles);
     return cudaGetLastError();
 }
 }  // namespace
