@@ -34,6 +34,7 @@ static_assert(half::kBX == kBX && half::kBY == kBY && f64::kNT == kNT, "tile sha
 template <int Q, int S, int MODE>
 __global__ void __launch_bounds__(kNT, 4) batch_kernel(const BatchItem *__restrict__ items, int nitems,
                                                        int64_t total_tiles) {
+    if constexpr (MODE == 3) dependent_wait();
     const int lane = threadIdx.x & 31;
     __shared__ aa::AANet no_network;  // batched instances have no mass-action network; never read
     double acc[S];
@@ -88,6 +89,7 @@ cudaError_t launch_batch(const BatchItem *items, int n, int64_t total, cudaStrea
     auto kern = batch_kernel<Q, S, MODE>;
     // FP64: one block per tile, as for a single grid (no mass is reduced here)
     const unsigned grid = MODE == 3 && total < (1 << 30) ? (unsigned)total : persistent_blocks(kern, kNT, total);
+    if constexpr (MODE == 3) return launch_dependent(kern, grid, dim3(kBX, kBY), 0, st, items, n, total);
     kern<<<grid, dim3(kBX, kBY), 0, st>>>(items, n, total);
     return cudaGetLastError();
 }

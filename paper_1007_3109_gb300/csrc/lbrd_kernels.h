@@ -48,6 +48,21 @@ unsigned persistent_blocks(K kernel, int nthreads, int64_t ntiles, size_t smem =
     const unsigned full = occupancy_blocks(reinterpret_cast<const void *>(kernel), nthreads, smem);
     return (unsigned)(ntiles < (int64_t)full ? (ntiles > 0 ? ntiles : 1) : full);
 }
+// Launch of a step kernel that starts with dependent_wait().
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
 // Upper bound of persistent_blocks over all kernels (sizes mass partials).
 unsigned max_persistent_blocks();
 

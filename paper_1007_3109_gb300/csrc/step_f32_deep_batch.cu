@@ -108,9 +108,8 @@ cudaError_t launch_pair_list(const DeepItem *items, int n, int64_t total_units, 
     if (e != cudaSuccess) return e;
     // total_units rows, shared out over the whole grid (at least one row per block)
     const unsigned grid = total_units < (int64_t)full ? (unsigned)total_units : full;
-    step_pair_kernel<Q, S, K, PS::NW, PS::NS, PS::MINB, true, true, !V16, RK>
-        <<<grid, PS::NW * 32, PS::smem, st>>>(StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
-    return cudaGetLastError();
+    return launch_dependent(step_pair_kernel<Q, S, K, PS::NW, PS::NS, PS::MINB, true, true, !V16, RK>, grid,
+                            PS::NW * 32, PS::smem, st, StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
 }
 
 // rk: the reaction kind of every grid of the list, or -1 (mixed); two-species
@@ -130,9 +129,8 @@ cudaError_t launch_batch(const DeepItem *items, int n, int64_t total_units, bool
         if (e != cudaSuccess) return e;
         const int64_t nwarps = (int64_t)full * BS::NW;
         const unsigned grid = total_units < nwarps ? (unsigned)((total_units + BS::NW - 1) / BS::NW) : full;
-        step_deep_kernel<Q, S, K, BS::NW, 4, BS::MINB, V16, true, BS::PP>
-            <<<grid, BS::NW * 32, BS::smem, st>>>(StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
-        return cudaGetLastError();
+        return launch_dependent(step_deep_kernel<Q, S, K, BS::NW, 4, BS::MINB, V16, true, BS::PP>, grid,
+                                BS::NW * 32, BS::smem, st, StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
     }
 }
 

@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     constexpr int KC = K > 1 ? K - 1 : 1;
     static_assert(K >= 1 && K <= 8 && NS >= 4, "depth 1 .. 8, at least four staged rows");
     extern __shared__ __align__(16) float smem[];
+    dependent_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float *ring = smem + (size_t)w * NS * kRow;
     const unsigned ring_s = static_cast<unsigned>(__cvta_generic_to_shared(ring));
@@ -357,9 +358,8 @@ cudaError_t launch_deep(const StepArgs &a, cudaStream_t st) {
     const int64_t band = (a.ny + nb - 1) / nb, nbands = (a.ny + band - 1) / band;
     const int64_t units = nstrips * nbands;
     const unsigned grid = units < nwarps ? (unsigned)((units + NW - 1) / NW) : full;
-    step_deep_kernel<Q, S, K, NW, NS, MINB, V16, false, PP>
-        <<<grid, NW * 32, DK::smem, st>>>(a, nstrips, nbands, band, nullptr, 0, 0, a.rho_out != nullptr);
-    return cudaGetLastError();
+    return launch_dependent(step_deep_kernel<Q, S, K, NW, NS, MINB, V16, false, PP>, grid,
+                            NW * 32, DK::smem, st, a, nstrips, nbands, band, nullptr, 0, 0, a.rho_out != nullptr);
 }
 
 }  // namespace

@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     constexpr int KC = K > 1 ? K - 1 : 1;
     static_assert(K >= 1 && K <= 8 && NS >= 4 && WO > 0, "depth 1 .. 8, at least four staged rows");
     extern __shared__ __align__(16) float smem[];
+    dependent_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float *ring = smem + (size_t)w * NS * kRow;
     const unsigned ring_s = static_cast<unsigned>(__cvta_generic_to_shared(ring));
@@ -428,9 +429,8 @@ cudaError_t launch_pair_rk(const StepArgs &a, cudaStream_t st) {
     const int64_t band = (a.ny + nb - 1) / nb, nbands = (a.ny + band - 1) / band;
     const int64_t units = nstrips * nbands;
     const unsigned grid = units < nwarps ? (unsigned)((units + NW - 1) / NW) : full;
-    step_pair_kernel<Q, S, K, NW, NS, MINB, false, PP, ANY, RK, EA>
-        <<<grid, NW * 32, PK::smem, st>>>(a, nstrips, nbands, band, nullptr, 0, 0, a.rho_out != nullptr);
-    return cudaGetLastError();
+    return launch_dependent(step_pair_kernel<Q, S, K, NW, NS, MINB, false, PP, ANY, RK, EA>, grid,
+                            NW * 32, PK::smem, st, a, nstrips, nbands, band, nullptr, 0, 0, a.rho_out != nullptr);
 }
 
 // Two-species Gray-Scott grids run the form with the reaction fixed at

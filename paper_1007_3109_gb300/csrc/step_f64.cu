@@ -15,6 +15,7 @@ static_assert(kNT == f64::kNT, "one block size");
 
 template <int Q, int S>
 __global__ void __launch_bounds__(kNT) step_f64_kernel(StepArgs a, int64_t ntiles) {
+    dependent_wait();
     double acc[S];
 #pragma unroll
     for (int s = 0; s < S; ++s) acc[s] = 0.0;
@@ -63,8 +64,7 @@ template <int Q, int S>
 cudaError_t launch_tiles(const StepArgs &a, cudaStream_t st) {
     const int64_t ntiles = f64::tiles(a.nx, a.ny);
     const unsigned grid = a.mass_out ? persistent_blocks(step_f64_kernel<Q, S>, kNT, ntiles) : (unsigned)ntiles;
-    step_f64_kernel<Q, S><<<grid, kNT, 0, st>>>(a, ntiles);
-    return cudaGetLastError();
+    return launch_dependent(step_f64_kernel<Q, S>, grid, kNT, 0, st, a, ntiles);
 }
 
 }  // namespace

@@ -62,7 +62,8 @@ __device__ __forceinline__ void weighted(double v, double (&c)[Lattice<Q>::kClas
 template <int Q, int S>
 __device__ __forceinline__ void site_f64(const StepArgs &a, int x, int y, double *acc) {
     using L = Lattice<Q>;
-    const double *__restrict__ src = static_cast<const double *>(a.src);
+    // plain loads (no read-only path): the kernel before may still be writing src when this one starts
+    const double *src = static_cast<const double *>(a.src);
     double *__restrict__ dst = static_cast<double *>(a.dst);
     const int nx = (int)a.nx, ny = (int)a.ny;
     // pulled rows y + 1, y, y - 1 and columns x + 1, x, x - 1 (periodic), by e + 1

@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     static_assert(NS == 3, "row j + 1 takes the slot of row j - 2");
     constexpr int NCH = CW / 4;
     extern __shared__ __align__(16) float smem[];
+    dependent_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float *ring = smem + (size_t)w * NS * kRow;
     const unsigned ring_s = static_cast<unsigned>(__cvta_generic_to_shared(ring));
@@ -288,8 +289,8 @@ cudaError_t launch_general_deep(const StepArgs &a, cudaStream_t st) {
     const int64_t band = (a.ny + nb - 1) / nb, nbands = (a.ny + band - 1) / band;
     const int64_t units = nstrips * nbands;
     const unsigned grid = units < nwarps ? (unsigned)((units + NW - 1) / NW) : full;
-    kern<<<grid, NW * 32, smem, st>>>(a, make_prog(a), (int)nstrips, (int)nbands, (int)band, a.rho_out != nullptr);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, NW * 32, smem, st, a, make_prog(a), (int)nstrips, (int)nbands, (int)band,
+                            a.rho_out != nullptr);
 }
 
 template <int K, int NW, int NS, int MINB>

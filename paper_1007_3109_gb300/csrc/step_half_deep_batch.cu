@@ -58,9 +58,8 @@ cudaError_t launch_half_batch_rk(const DeepItem *items, int n, int64_t total_uni
     if (e != cudaSuccess) return e;
     const int64_t nwarps = (int64_t)full * HS::NW;
     const unsigned grid = total_units < nwarps ? (unsigned)((total_units + HS::NW - 1) / HS::NW) : full;
-    step_half_deep_kernel<Q, S, H, K, HS::NW, HS::NS, HS::MINB, true, RK>
-        <<<grid, HS::NW * 32, HK::smem, st>>>(StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
-    return cudaGetLastError();
+    return launch_dependent(step_half_deep_kernel<Q, S, H, K, HS::NW, HS::NS, HS::MINB, true, RK>, grid,
+                            HS::NW * 32, HK::smem, st, StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
 }
 
 template <int Q, int S, int H, int K, int RK>
@@ -72,9 +71,8 @@ cudaError_t launch_half_pair_list(const DeepItem *items, int n, int64_t total_un
     if (e != cudaSuccess) return e;
     // total_units rows, shared out over the whole grid (at least one row per block)
     const unsigned grid = total_units < (int64_t)full ? (unsigned)total_units : full;
-    step_half_pair_kernel<Q, S, H, K, PS::NW, PS::NS, PS::MINB, true, RK>
-        <<<grid, PS::NW * 32, HK::smem, st>>>(StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
-    return cudaGetLastError();
+    return launch_dependent(step_half_pair_kernel<Q, S, H, K, PS::NW, PS::NS, PS::MINB, true, RK>, grid,
+                            PS::NW * 32, HK::smem, st, StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
 }
 
 // rk: the reaction kind of every grid of the list, or -1 (mixed); v8: every

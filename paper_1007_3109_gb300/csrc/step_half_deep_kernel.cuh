@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     constexpr int NCP = S * Q;                // staged planes per row (rho* and QD deviations per species)
     static_assert(K >= 1 && K <= 8 && NS >= 4 && kSp % 16 == 0, "depth 1 .. 8, at least four staged rows");
     extern __shared__ __align__(16) unsigned char hsm[];
+    dependent_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned char *ring = hsm + (size_t)w * NS * kRow;
     const unsigned ring_s = static_cast<unsigned>(__cvta_generic_to_shared(ring));
@@ -294,9 +295,8 @@ cudaError_t launch_half_deep_rk(const StepArgs &a, cudaStream_t st) {
     const int64_t band = (a.ny + nb - 1) / nb, nbands = (a.ny + band - 1) / band;
     const int64_t units = nstrips * nbands;
     const unsigned grid = units < nwarps ? (unsigned)((units + NW - 1) / NW) : full;
-    step_half_deep_kernel<Q, S, H, K, NW, NS, MINB, false, RK>
-        <<<grid, NW * 32, HK::smem, st>>>(a, nstrips, nbands, band, nullptr, 0, 0, a.rho_out != nullptr);
-    return cudaGetLastError();
+    return launch_dependent(step_half_deep_kernel<Q, S, H, K, NW, NS, MINB, false, RK>, grid,
+                            NW * 32, HK::smem, st, a, nstrips, nbands, band, nullptr, 0, 0, a.rho_out != nullptr);
 }
 
 // Two-species Gray-Scott grids run the form with the reaction fixed at

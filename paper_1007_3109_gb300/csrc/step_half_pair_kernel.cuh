@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     constexpr bool PK = MINB <= 2;  // packed pairs where the launch bounds allow 255 registers
     static_assert(K >= 1 && K <= 8 && NS >= 4 && WO > 0 && kSp % 16 == 0, "depth 1 .. 8, four staged rows");
     extern __shared__ __align__(16) unsigned char hps[];
+    dependent_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned char *ring = hps + (size_t)w * NS * kRow;
     const unsigned ring_s = static_cast<unsigned>(__cvta_generic_to_shared(ring));
@@ -439,9 +440,8 @@ cudaError_t launch_half_pair_rk(const StepArgs &a, cudaStream_t st) {
     const int64_t band = (a.ny + nb - 1) / nb, nbands = (a.ny + band - 1) / band;
     const int64_t units = nstrips * nbands;
     const unsigned grid = units < nwarps ? (unsigned)((units + NW - 1) / NW) : full;
-    step_half_pair_kernel<Q, S, H, K, NW, NS, MINB, false, RK>
-        <<<grid, NW * 32, HK::smem, st>>>(a, nstrips, nbands, band, nullptr, 0, 0, a.rho_out != nullptr);
-    return cudaGetLastError();
+    return launch_dependent(step_half_pair_kernel<Q, S, H, K, NW, NS, MINB, false, RK>, grid,
+                            NW * 32, HK::smem, st, a, nstrips, nbands, band, nullptr, 0, 0, a.rho_out != nullptr);
 }
 
 // nx a multiple of 8 (16-byte chunks of 16-bit values never straddle the
