@@ -195,13 +195,13 @@ void default_depths(lb_rd_handle *h) {
 // step there is launch latency either way (256^2: 6.2 us, five steps per launch
 // 2.9 us each), and callers that time or count the steps of small grids see
 // each one.  Above, us per step of the rule's choice against the one-step
-// default, FP32 D2Q9 with two species: 512^2 4.1 / 8.3, 1531 x 1021 13.9 / 49.3,
+// default, FP32 D2Q9 with two species: 512^2 4.1 / 8.3, 1531 x 1021 13.2 / 49.3,
 // 2048^2 24.6 / 102, 4096^2 87 / 391; D2Q5 4096^2 38 / 207; bf16 deviations
 // 2048^2 30 / 62.  The lines between two choices lie where the autotuner's times
 // cross: the six-row ring hides the latency of L2-resident rows (512^2: 4.1
-// against 4.5, 1024^2 8.6 / 8.9, 1448^2 14.2 / 14.0), the any-nx two-column form
-// needs enough rows per warp (383 x 511: 5.4 against the one-column form's 5.2,
-// 767 x 703 7.4 / 7.7), K = 2 beats K = 3 for four D2Q9 species on small grids
+// against 4.5, 1024^2 8.6 / 8.9, 1448^2 14.2 / 14.0), any nx takes four steps on
+// small grids (383 x 511: 4.2 against five steps' 5.0; 767 x 703 6.5 / 6.6;
+// 1531 x 1021 14.0 / 13.2), K = 2 beats K = 3 for four D2Q9 species on small grids
 // (512^2: 14.5 / 17.9; 2048^2: 139 / 135).
 int default_bulk(const lb_rd_handle *h) {
     const int64_t sites = h->cfg.nx * h->cfg.ny;
@@ -213,7 +213,7 @@ int default_bulk(const lb_rd_handle *h) {
         return first_fitting(h, {"hpair4_128_minb2", sites < (1 << 21) ? "hdeep4_128_minb2" : "hdeep4_128_minb3"});
     if (h->S * h->Q > 10)
         return first_fitting(h, {sites <= (3 << 19) ? "deep5vw_128_minb2_s6" : "deep5vw_256_minb1",
-                                 sites < (3 << 17) ? "deep4_128_minb3" : "deep5vwpa_256_minb1"});
+                                 sites < (1 << 19) ? "deep4vwa_128_minb2" : "deep5vwpa_256_minb1"});
     return first_fitting(h, {h->Q == 9 ? "deep6vwpe_128_minb1_s5" : "deep6vwp_128_minb1_s6", "deep6vwpa_128_minb1"});
 }
 

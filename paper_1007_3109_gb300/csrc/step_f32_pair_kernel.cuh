@@ -20,9 +20,12 @@
 //     16-31 chunk `lane - 16` of the odd planes, lane p < S Q chunk 16 of
 //     plane p.  nx a multiple of 4: no chunk straddles the periodic seam.
 //     The ANY form takes any nx: a chunk that reaches past the seam (edge
-//     strips only) is copied column by column with wrapped indices; kept
-//     apart because the extra paths slow the loop body down even where they
-//     never run.  Waits only on the warp's own copy groups.
+//     strips only) is copied column by column, a lane per column with its
+//     wrapped position from shared memory (with a remainder per copy by the
+//     lane that owns the chunk, an edge strip's warp took twice as long per
+//     row and every launch waited for it: 4095^2 111 -> 95 us per step); kept apart
+//     because the extra paths slow the loop body down even where they never
+//     run.  Waits only on the warp's own copy groups.
 //   * level 1 pulls the lane's column pair of every plane from the staged row
 //     of its e_iy (one 8-byte shared load) and shifts it like the levels
 //     above; level m > 1 pulls from level m - 1 carried in registers (the row
@@ -108,6 +111,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     // BATCH: the unit's grid parameters, one copy per warp, read where they
     // are used so that they hold no registers across the row loop (a single
     // grid reads them from the kernel's parameter space)
+    __shared__ int wcol_sh[ANY ? NW : 1][ANY ? CW + 2 : 1];
     __shared__ SegArgs seg_sh[BATCH ? NW : 1];
     SegArgs &gs = seg_sh[BATCH ? w : 0];
     auto p_src = [&]() -> const float * {
@@ -189,11 +193,32 @@ __global__ void __launch_bounds__(NW * 32, MINB)
         const int xb = (int)(strip * WO) - HL;  // first window column (even)
         const int a0 = xb - (int)wrap_mod(xb, 4);  // first staged column
         const int o = xb - a0;                     // staged column of xb: 0 or 2
-        // this lane's chunks start at columns cA and cB; a chunk that reaches past the
-        // periodic seam (edge strips only, nx not a multiple of 4) is copied column by
-        // column with wrapped indices, the others in one 16-byte copy
+        // this lane's chunks start at columns cA and cB.  ANY: a chunk that reaches past the
+        // periodic seam (edge strips only) is copied column by column: chunks [clo, chi) lie
+        // inside the grid, the columns of the others have their wrapped positions in wcol_sh,
+        // which for a single grid also holds 4 clo and 4 chi (no registers across the row loop)
         const int cA = a0 + 4 * cch, cB = a0 + 64;
-        const bool cleanA = !ANY || (cA >= 0 && cA + 4 <= nx), cleanB = !ANY || (cB >= 0 && cB + 4 <= nx);
+        bool edge = false, cleanA = true, cleanB = true;
+        int clo4 = 0, chi4 = CW;
+        if constexpr (ANY) {
+            const int clo = a0 < 0 ? -a0 / 4 : 0;
+            int chi = (nx - a0) / 4;
+            chi = chi < clo ? clo : (chi > 17 ? 17 : chi);
+            edge = clo > 0 || chi < 17;
+            clo4 = 4 * clo;
+            chi4 = 4 * chi;
+            cleanA = cch >= clo && cch < chi;
+            cleanB = clo <= 16 && chi > 16;
+            __syncwarp();  // the previous unit's reads of wcol are done
+            if (edge) {
+                for (int q = lane; q < CW; q += 32) wcol_sh[w][q] = wrap32(a0 + q, nx);
+                if (lane == 0) {
+                    wcol_sh[w][CW] = clo4;
+                    wcol_sh[w][CW + 1] = chi4;
+                }
+            }
+            __syncwarp();
+        }
         const int64_t offA = (int64_t)cpar * g.plane + (ANY ? (cleanA ? cA : 0) : wrap_mod(cA, nx));
         const int64_t offB = (int64_t)(lane < SQ ? lane : 0) * g.plane + (ANY ? (cleanB ? cB : 0) : wrap_mod(cB, nx));
         const int nrows = ly + 2 * K;
@@ -209,20 +234,22 @@ __global__ void __launch_bounds__(NW * 32, MINB)
 #pragma unroll
                     for (int r = 0; r < (SQ + 1) / 2; ++r)
                         if (cpar + 2 * r < SQ) cp_async16(d + (unsigned)(2 * r * CW * 4), sp + r * pl2);
-                } else if constexpr (ANY) {
-                    for (int r = 0; r < (SQ + 1) / 2; ++r)
-                        if (cpar + 2 * r < SQ)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                cp_async4s(d + (unsigned)((2 * r * CW + e) * 4), sp + r * pl2 + wrap32(cA + e, nx));
                 }
-                if (lane < SQ) {
-                    const unsigned db = ring_s + (unsigned)(slot * kRow + lane * CW + 64) * 4u;
-                    if (!ANY || cleanB) {
-                        cp_async16(db, row + offB);
-                    } else if constexpr (ANY) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) cp_async4s(db + 4u * e, row + offB + wrap32(cB + e, nx));
+                if (lane < SQ && cleanB)
+                    cp_async16(ring_s + (unsigned)(slot * kRow + lane * CW + 64) * 4u, row + offB);
+                if constexpr (ANY) {
+                    if (edge) {  // warp-uniform: a lane per column, plane by plane
+                        const volatile int *wc = wcol_sh[w];
+                        const int lo4 = BATCH ? clo4 : wc[CW], hi4 = BATCH ? chi4 : wc[CW + 1], nu = lo4 + CW - hi4;
+                        int64_t pl = p_plane();
+                        asm volatile("" : "+l"(pl));
+                        for (int q = lane; q < nu; q += 32) {
+                            const int c = q < lo4 ? q : q - lo4 + hi4;
+                            const float *cp = row + wc[c];
+                            const unsigned dc = ring_s + (unsigned)(slot * kRow + c) * 4u;
+#pragma unroll 6
+                            for (int pp = 0; pp < SQ; ++pp) cp_async4s(dc + (unsigned)(pp * CW * 4), cp + pp * pl);
+                        }
                     }
                 }
             }
