@@ -324,11 +324,11 @@ LB_RD_API int lb_rd_batch_set_graph(lb_rd_batch *b, int32_t steps_per_graph);
  * instances are FP32 with two state copies and nx a multiple of 256; other
  * values >= 2 (and 2 otherwise) run the depth-K kernel over the rows of all
  * instances (FP32, two state copies, any nx; bitwise the same as
- * K single steps; for K <= 5 (D2Q9) or 6 (D2Q5) its form with two columns per
- * lane; the default for such batches: 5 for D2Q9, 6 for D2Q5); 16-bit
- * deviation storage runs its own depth-K kernels, K = 2 .. 5 (the
- * two-column form when every nx is a multiple of 8, default 5; else default
- * 4).
+ * K single steps; for K <= 6 its form with two columns per lane; the default
+ * for such batches: 6, or 5 for D2Q9 with one species or with fewer than 1.5 M
+ * sites in all (1.5 * 2^20)); 16-bit
+ * deviation storage runs its own depth-K kernels, K = 2 .. 5, default 4 (the
+ * two-column form when every nx is a multiple of 8).
  * EINVAL if neither applies.  1: one step per launch (the default for other
  * batches).  The graphs of lb_rd_batch_set_graph hold steps_per_graph / K
  * launches.  Synchronises the batch's stream. */
@@ -349,8 +349,8 @@ LB_RD_API int lb_rd_batch_get_time(const lb_rd_batch *b, int64_t *t, int64_t *la
  * Resident requests advance together, steps_per_tick steps at a time (fewer
  * when a request finishes sooner), by launches of the batched kernels over
  * all of them: for FP32 and 16-bit deviation requests with two state copies,
- * tick / K launches of the depth-K kernel (K as the batches' default: 5 for
- * D2Q9 and 6 for D2Q5 in FP32; 5 or 4 in 16-bit storage) and one launch of the
+ * tick / K launches of the depth-K kernel (K as a batch of them would take by
+ * default) and one launch of the
  * tick % K
  * steps left (a single step if one is left), otherwise one launch per step;
  * the last launch of a tick also writes the densities.  Requests that arrive

@@ -518,8 +518,8 @@ class Batch:
 
     def set_steps_per_launch(self, k):
         """Time steps per batched launch: 1, 2 (two-step kernel, every nx a
-        multiple of 256) or 4, 5, 6, 8 (depth-K kernel; FP32 batches with two
-        state copies default to 6 for D2Q9, 4 for D2Q5).  Bitwise the same
+        multiple of 256) or 2 .. 8 (depth-K kernel; FP32 batches with two state
+        copies default to 5 or 6 by size).  Bitwise the same
         results for every choice."""
         lb_rd_batch_set_steps_per_launch(self.b, k)
         return self

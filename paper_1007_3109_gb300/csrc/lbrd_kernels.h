@@ -177,8 +177,8 @@ struct TbwItem {
 int batch_tb2_strip();
 cudaError_t launch_batch_tb2(const TbwItem *items, int n, int64_t total_units, int Q, int S, cudaStream_t st);
 // Batched K-step launches (K = 2 .. 8; FP32, two state copies): the depth-K
-// kernel over the (band, strip) units of a list of grids (for K <= 5 (D2Q9)
-// or 6 (D2Q5) its two-column form).  The one-column form's units of item k
+// kernel over the (band, strip) units of a list of grids (for K <= 6 its
+// two-column form).  The one-column form's units of item k
 // are [unit_begin, unit_begin + nstrips * ceil(ny / band)), strips of the
 // kernel's 34 - 2K output columns fastest; the two-column form shares out the
 // list's rows (list_rows.cuh).  batch_deep_plan fills the descriptors (one-column
@@ -206,10 +206,12 @@ int batch_half_default_k();
 cudaError_t launch_batch_half_deep(int K, int Q, int S, int half_kind, const DeepItem *items, int n,
                                    int64_t total_units, bool emit, int rk, bool v8, cudaStream_t st);
 bool batch_deep_depth_ok(int K);
-// Default steps per launch of a list of grids: 5 (D2Q9) / 6 (D2Q5), the
-// fastest two-column forms over a list (the grid's parameters read from a
-// per-warp shared copy where they are used).
-int batch_deep_default_k(int Q);
+// Default steps per launch of a list of `sites` sites: 6, the deepest two-column
+// form, which moves the state least often; 5 for D2Q9 lists of one species or of
+// fewer than 1.5 M sites, where the rows that fill the levels weigh more (five
+// grids of sides 190 .. 500: 9.3 us per step at K = 5, 9.4 at 6; 9 x 512^2 15.2 /
+// 14.3; 256 x 256^2 98.6 / 90.7).
+int batch_deep_default_k(int Q, int S, int64_t sites);
 int64_t batch_deep_plan(int K, int Q, int S, bool v16, DeepItem *items, int n);
 cudaError_t launch_batch_deep(int K, int Q, int S, bool v16, const DeepItem *items, int n, int64_t total_units,
                               bool emit, int rk, cudaStream_t st);

@@ -7,7 +7,7 @@
 // fill the levels once per segment.  Short lists, where that second fill would
 // cost more than uneven parts, are cut into bands of one height instead, no
 // more bands than workers: 12 uneven grids of sides 64 .. 1024 run at 28.9 us
-// per step so and at 30.8 in equal parts, 9 x 512^2 at 15.3 and 16.8.
+// per step so and at 30.8 in equal parts, 9 x 512^2 at 15.3 and 16.8 (K = 5).
 //
 // A worker is a block, whose NW warps walk NW adjacent strips side by side
 // (group size NW), or a warp (group size 1).  Strips of consecutive grids of
@@ -28,7 +28,7 @@ namespace {
 // Sites of a list above which the warps of a block meet every four rows (FP32
 // D2Q9): the halo columns that two strips share are then read while they are in
 // L2.  40 uneven grids of sides up to 2048 (60 M sites): 422 -> 388 us per
-// step; 256 grids of 255^2: 137 -> 127; 256^2: no change.  Lists that sit
+// step (K = 5); 256 grids of 255^2: 137 -> 127; 256^2: no change.  Lists that sit
 // closer to L2 lose a little instead (9 x 512^2, 2.4 M sites: 16.7 -> 17.3).
 constexpr int64_t kLockstepSites = 8 << 20;
 

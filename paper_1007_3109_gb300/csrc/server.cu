@@ -8,7 +8,7 @@
 //   2. advances every resident request by one tick of up to steps_per_tick
 //      steps (never past the earliest finishing request): FP32 requests with
 //      two state copies by K-step launches of the depth-K kernel over all
-//      resident requests (K = 5 for D2Q9, 6 for D2Q5: the two-column form;
+//      resident requests (K = 5 or 6 by their size: the two-column form;
 //      16-bit deviation storage its own kernel, K = 4) and one shorter
 //      depth-K launch for the steps left (a single step if one is left),
 //      other requests one batched launch per step; the tick's last launch
@@ -270,7 +270,9 @@ void run_tick(lb_rd_server *s) {
     for (Request *r : act) v16 = v16 && r->cfg.nx % 4 == 0 && r->pitch % 4 == 0;
     for (Request *r : act) v8 = v8 && r->cfg.nx % 8 == 0 && r->pitch % 8 == 0;
     const bool half = s->mode == 1 || s->mode == 2;  // 16-bit deviation storage: its own depth-K kernels
-    const int K = half ? lbrd::batch_half_default_k() : lbrd::batch_deep_default_k(s->Q);
+    int64_t sites = 0;
+    for (Request *r : act) sites += r->cfg.nx * r->cfg.ny;
+    const int K = half ? lbrd::batch_half_default_k() : lbrd::batch_deep_default_k(s->Q, s->cfg.nspecies, sites);
     const bool deep = (s->mode == 0 || half) && !any_inplace && tick >= 2;
     int64_t n_multi = deep ? tick / K : 0;
     int rem = deep ? (int)(tick % K) : 0;  // steps of the depth-r launch (0: none)

@@ -134,6 +134,11 @@ const F32Variant kF32Variants[] = {
     {"deep5vwpa_256_minb1", 256, 5, 1, 4, 5, 1},
     // two columns per lane, a row staged as soon as level 1 has read the oldest one: deep<K>vw[p]e_
     {"deep6vwpe_128_minb1_s5", 128, 6, 1, 4, 6, 4},
+    // two columns per lane: three rows staged ahead; one level's rows in shared memory: deep<K>vwm[a]_
+    {"deep4vwp_128_minb1_s6", 128, 4, 1, 4, 4, 4},
+    {"deep6vwm_256_minb1", 256, 6, 1, 4, 6, 4},
+    {"deep6vwm_128_minb2", 128, 6, 2, 4, 6, 4},
+    {"deep6vwma_256_minb1", 256, 6, 1, 4, 6, 1},
 };
 const int kF32VariantCount = sizeof(kF32Variants) / sizeof(kF32Variants[0]);
 

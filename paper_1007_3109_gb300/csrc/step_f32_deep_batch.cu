@@ -9,57 +9,27 @@ namespace lbrd {
 namespace {
 
 // Two columns per lane (step_f32_pair_kernel.cuh) where that form is the
-// faster one: depths whose carried levels fit the register file without
-// heavy spills (K <= 5 for D2Q9, K <= 6 for D2Q5); its any-nx form unless
-// every grid has nx a multiple of 4.  Four warps, the pulls from earlier rows
-// first, five staged rows below K = 5 and for D2Q5 (whose smaller rows leave
-// L1 its share with two rows staged ahead).
-template <int Q, int K, bool V16>
+// faster one: depths whose carried levels fit the register file (K <= 5), and
+// K = 6, for two D2Q9 species with level 4's rows in shared memory; its any-nx
+// form unless every grid has nx a multiple of 4.  Four warps, the pulls from
+// earlier rows first (not with a level in shared memory), five staged rows below
+// K = 5 and for D2Q5 (whose smaller rows leave L1 its share with two rows staged
+// ahead).
+template <int K>
 struct UsePair {
-    static constexpr bool value = Q == 9 ? K <= 5 : K <= 6;
+    static constexpr bool value = K <= 6;
 };
 template <int Q, int S, int K, bool V16, int RK = -1>
-struct PairShape
-    : PairKernel<Q, S, K, 4, (K < 5 || Q == 5 ? 5 : 4), (K == 6 ? 1 : 2), true, true, !V16, RK> {
-    static constexpr int NW = 4, NS = K < 5 || Q == 5 ? 5 : 4, MINB = K == 6 ? 1 : 2;
+struct PairShape {
+    static constexpr int NW = 4, NS = K < 5 || Q == 5 ? 5 : 4, SML = K == 6 && Q * S > 10 ? 8 : 0;
+    static constexpr int MINB = K == 6 && SML == 0 ? 1 : 2;
+    using Kernel = PairKernel<Q, S, K, NW, NS, MINB, true, SML == 0, !V16, RK, false, SML>;
 };
 
-// Batched launch shapes per K: the single-grid choices (K = 4, 5: six warps,
-// two blocks per SM; K = 6, 7, 8: four warps, two blocks per SM; K = 5, 7, 8
-// with the pulls from earlier rows first; K = 2, 3, which cover the last steps
-// of a call or a tick: four warps, four and three blocks per SM).
+// One column per lane, K = 7 and 8: four warps, two blocks per SM, the pulls from
+// earlier rows first.
 template <int Q, int S, int K, bool V16>
 struct BatchShape;
-template <int Q, int S, bool V16>
-struct BatchShape<Q, S, 2, V16> : DeepKernel<Q, S, 2, 4, 4, 4, V16, true> {
-    static constexpr int NW = 4;
-    static constexpr int MINB = 4;
-    static constexpr bool PP = false;
-};
-template <int Q, int S, bool V16>
-struct BatchShape<Q, S, 3, V16> : DeepKernel<Q, S, 3, 4, 4, 3, V16, true> {
-    static constexpr int NW = 4;
-    static constexpr int MINB = 3;
-    static constexpr bool PP = false;
-};
-template <int Q, int S, bool V16>
-struct BatchShape<Q, S, 4, V16> : DeepKernel<Q, S, 4, 6, 4, 2, V16, true> {
-    static constexpr int NW = 6;
-    static constexpr int MINB = 2;
-    static constexpr bool PP = false;
-};
-template <int Q, int S, bool V16>
-struct BatchShape<Q, S, 5, V16> : DeepKernel<Q, S, 5, 6, 4, 2, V16, true, true> {
-    static constexpr int NW = 6;
-    static constexpr int MINB = 2;
-    static constexpr bool PP = true;
-};
-template <int Q, int S, bool V16>
-struct BatchShape<Q, S, 6, V16> : DeepKernel<Q, S, 6, 4, 4, 2, V16, true> {
-    static constexpr int NW = 4;
-    static constexpr int MINB = 2;
-    static constexpr bool PP = false;
-};
 template <int Q, int S, bool V16>
 struct BatchShape<Q, S, 7, V16> : DeepKernel<Q, S, 7, 4, 4, 2, V16, true, true> {
     static constexpr int NW = 4;
@@ -75,14 +45,14 @@ struct BatchShape<Q, S, 8, V16> : DeepKernel<Q, S, 8, 4, 4, 2, V16, true, true> 
 
 template <int Q, int S, int K, bool V16>
 int64_t plan_batch(DeepItem *items, int n) {
-    constexpr bool pair = UsePair<Q, K, V16>::value;
+    constexpr bool pair = UsePair<K>::value;
     constexpr int WO = pair ? PairGeom<K>::WO : 34 - 2 * K;
     int NW = 0;
     unsigned full = 0;
     cudaError_t ge;
     if constexpr (pair) {  // only the kernels a list can run are instantiated
         NW = PairShape<Q, S, K, V16>::NW;
-        ge = PairShape<Q, S, K, V16>::get(&full);
+        ge = PairShape<Q, S, K, V16>::Kernel::get(&full);
     } else {
         NW = BatchShape<Q, S, K, V16>::NW;
         ge = BatchShape<Q, S, K, V16>::get(&full);
@@ -104,12 +74,13 @@ template <int Q, int S, int K, bool V16, int RK>
 cudaError_t launch_pair_list(const DeepItem *items, int n, int64_t total_units, bool emit, cudaStream_t st) {
     using PS = PairShape<Q, S, K, V16, RK>;
     unsigned full = 0;
-    cudaError_t e = PS::get(&full);
+    cudaError_t e = PS::Kernel::get(&full);
     if (e != cudaSuccess) return e;
     // total_units rows, shared out over the whole grid (at least one row per block)
     const unsigned grid = total_units < (int64_t)full ? (unsigned)total_units : full;
-    return launch_dependent(step_pair_kernel<Q, S, K, PS::NW, PS::NS, PS::MINB, true, true, !V16, RK>, grid,
-                            PS::NW * 32, PS::smem, st, StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
+    return launch_dependent(step_pair_kernel<Q, S, K, PS::NW, PS::NS, PS::MINB, true, PS::SML == 0, !V16, RK, false,
+                                             PS::SML>,
+                            grid, PS::NW * 32, PS::Kernel::smem, st, StepArgs{}, 0, 0, 0, items, n, total_units, emit ? 1 : 0);
 }
 
 // rk: the reaction kind of every grid of the list, or -1 (mixed); two-species
@@ -118,7 +89,7 @@ cudaError_t launch_pair_list(const DeepItem *items, int n, int64_t total_units, 
 // instantiation spilled more and ran K = 5 at 0.6x the speed of the other).
 template <int Q, int S, int K, bool V16>
 cudaError_t launch_batch(const DeepItem *items, int n, int64_t total_units, bool emit, int rk, cudaStream_t st) {
-    if constexpr (UsePair<Q, K, V16>::value) {
+    if constexpr (UsePair<K>::value) {
         if constexpr (S == 2 && V16)
             if (rk == kGrayScott) return launch_pair_list<Q, S, K, V16, kGrayScott>(items, n, total_units, emit, st);
         return launch_pair_list<Q, S, K, V16, -1>(items, n, total_units, emit, st);
@@ -164,7 +135,7 @@ cudaError_t launch_v(int Q, int S, bool v16, const DeepItem *items, int n, int64
 
 bool batch_deep_depth_ok(int K) { return K >= 2 && K <= 8; }
 
-int batch_deep_default_k(int Q) { return Q == 9 ? 5 : 6; }
+int batch_deep_default_k(int Q, int S, int64_t sites) { return Q == 9 && (S == 1 || sites < (3 << 19)) ? 5 : 6; }
 
 int64_t batch_deep_plan(int K, int Q, int S, bool v16, DeepItem *items, int n) {
     switch (K) {

@@ -79,13 +79,29 @@ struct PairGeom {
     static constexpr int WO = 64 - 2 * HL;      // output columns per warp, even
 };
 
+// Rows of one level carried in shared memory, private to each lane: the previous
+// row's e_iy = 0 components, then the e_iy = +1 components of the two rows before
+// (row j takes the place of row j - 2), each a lane's two columns.
+template <int Q, int S>
+struct PairCarry {
+    static constexpr int nE = 3 * S, nP = (Q == 9 ? 3 : 1) * S;
+    static constexpr int kWarp = (nE + 2 * nP) * 32;  // float2 per warp and level
+};
+
 // ANY: grids of any nx (the seam chunks copied column by column, the last
 // column of an odd nx stored alone); otherwise nx must be a multiple of 4.
 // RK >= 0: the grid's reaction kind, fixed at compile time.  EA: a row is
 // staged as soon as level 1 has read the oldest staged row, whose slot it
 // takes: NS - 2 rows in flight instead of NS - 3, in the same ring.
+// SML: bit m - 1 set: level m's rows are carried in shared memory instead of
+// registers (not with PP).  At K = 6 the five carried levels of D2Q9 with two
+// species need 180 registers; with level 4 in shared memory (4.6 KB per warp, 24
+// eight-byte accesses per row and no moves between rows) the kernel spills 44
+// bytes instead of 144 and moves the state once per six steps: 8192^2 342 -> 317
+// us per step against K = 5, 2048^2 23.9 -> 22.3.  Levels 2 .. 5 measure alike;
+// two levels want a three-row ring (337 us: a row ahead is not enough).
 template <int Q, int S, int K, int NW, int NS, int MINB, bool BATCH, bool PP, bool ANY = false, int RK = -1,
-          bool EA = false>
+          bool EA = false, int SML = 0>
 __global__ void __launch_bounds__(NW * 32, MINB)
     step_pair_kernel(StepArgs a, int64_t nstrips, int64_t nbands, int64_t band, const DeepItem *__restrict__ items,
                      int nitems, int64_t total_units, int emit) {
@@ -103,6 +119,10 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float *ring = smem + (size_t)w * NS * kRow;
     const unsigned ring_s = static_cast<unsigned>(__cvta_generic_to_shared(ring));
+    using PC = PairCarry<Q, S>;
+    static_assert(SML == 0 || !PP, "levels in shared memory: without the pulls-first order");
+    constexpr int kSM = __builtin_popcount(SML);
+    float2 *carry = reinterpret_cast<float2 *>(smem + (size_t)NW * NS * kRow) + (size_t)w * kSM * PC::kWarp + lane;
     SegArgs g;
     if (!BATCH) {
         load_seg(a, g);
@@ -136,7 +156,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     };
     // relaxation and reaction constants of the collisions
     auto p_coll = [&]() -> SegArgs {
-        if constexpr (BATCH) {
+        if constexpr (BATCH && SML == 0) {
             SegArgs c;
             c.omega[0] = __uint_as_float(lds_v32(&gs.omega[0]));
             c.omega[1] = __uint_as_float(lds_v32(&gs.omega[1]));
@@ -149,10 +169,11 @@ __global__ void __launch_bounds__(NW * 32, MINB)
             return g;
         }
     };
-    // lists of two-species D2Q9 grids: the species of a site packed (256 x 256^2 at K = 5: 98.0 against
+    // lists of two-species D2Q9 grids and the kernels with a level in shared memory, which are
+    // bound by instruction issue: the species of a site packed (lists, 256 x 256^2 at K = 5: 98.0 against
     // 99.4 us per step, 256 x 255^2 137 / 145, 9 x 512^2 16.7 / 17.6; D2Q5 and single grids gain nothing)
     auto collide = [](const SegArgs &cg, float(&f0)[S][Q], float(&f1)[S][Q], float(&rho0)[S], float(&rho1)[S]) {
-        if constexpr (BATCH && Q == 9 && S == 2) collide_pair_species<Q, RK>(cg, f0, f1, rho0, rho1);
+        if constexpr ((BATCH || SML) && Q == 9 && S == 2) collide_pair_species<Q, RK>(cg, f0, f1, rho0, rho1);
         else collide_pair<Q, S, RK>(cg, f0, f1, rho0, rho1);
     };
     double acc[S];
@@ -349,24 +370,38 @@ __global__ void __launch_bounds__(NW * 32, MINB)
                         }
                 } else {
                     float h0[S][Q], h1[S][Q];
+                    const bool in_smem = (SML >> (m - 1)) & 1;
+                    float2 *cs = carry + __builtin_popcount(SML & ((1 << (m - 1)) - 1)) * PC::kWarp;
+                    float2 *cp = cs + (PC::nE + (j & 1) * PC::nP) * 32;
+                    int ie = 0, ip = 0;
 #pragma unroll
                     for (int s = 0; s < S; ++s)
 #pragma unroll
                         for (int i = 0; i < Q; ++i) {
-                            const float v0 = L::ey(i) < 0    ? f0[s][i]
-                                             : L::ey(i) == 0 ? E0[m - 1][0][s][i]
-                                                             : P2[m - 1][0][s][i];
-                            const float v1 = L::ey(i) < 0    ? f1[s][i]
-                                             : L::ey(i) == 0 ? E0[m - 1][1][s][i]
-                                                             : P2[m - 1][1][s][i];
+                            float v0, v1;
+                            if (L::ey(i) < 0) {
+                                v0 = f0[s][i];
+                                v1 = f1[s][i];
+                            } else if (in_smem) {
+                                const float2 v = L::ey(i) == 0 ? cs[32 * ie++] : cp[32 * ip++];
+                                v0 = v.x;
+                                v1 = v.y;
+                            } else {
+                                v0 = L::ey(i) == 0 ? E0[m - 1][0][s][i] : P2[m - 1][0][s][i];
+                                v1 = L::ey(i) == 0 ? E0[m - 1][1][s][i] : P2[m - 1][1][s][i];
+                            }
                             h0[s][i] = L::ex(i) > 0 ? __shfl_up_sync(kFullMask, v1, 1) : (L::ex(i) < 0 ? v1 : v0);
                             h1[s][i] = L::ex(i) > 0 ? v0 : (L::ex(i) < 0 ? __shfl_down_sync(kFullMask, v0, 1) : v1);
                         }
+                    ie = ip = 0;
 #pragma unroll
                     for (int s = 0; s < S; ++s)
 #pragma unroll
                         for (int i = 0; i < Q; ++i) {
-                            if (L::ey(i) > 0) {
+                            if (in_smem) {
+                                if (L::ey(i) > 0) cp[32 * ip++] = make_float2(f0[s][i], f1[s][i]);
+                                else if (L::ey(i) == 0) cs[32 * ie++] = make_float2(f0[s][i], f1[s][i]);
+                            } else if (L::ey(i) > 0) {
                                 P2[m - 1][0][s][i] = P1[m - 1][0][s][i];
                                 P2[m - 1][1][s][i] = P1[m - 1][1][s][i];
                                 P1[m - 1][0][s][i] = f0[s][i];
@@ -425,11 +460,12 @@ __global__ void __launch_bounds__(NW * 32, MINB)
 }
 
 template <int Q, int S, int K, int NW, int NS, int MINB, bool BATCH, bool PP = false, bool ANY = false, int RK = -1,
-          bool EA = false>
+          bool EA = false, int SML = 0>
 struct PairKernel {
-    static constexpr size_t smem = (size_t)NW * NS * S * Q * 68 * sizeof(float);
+    static constexpr size_t smem =
+        NW * ((size_t)NS * S * Q * 68 * sizeof(float) + __builtin_popcount(SML) * PairCarry<Q, S>::kWarp * sizeof(float2));
     static cudaError_t get(unsigned *full) {
-        auto kern = step_pair_kernel<Q, S, K, NW, NS, MINB, BATCH, PP, ANY, RK, EA>;
+        auto kern = step_pair_kernel<Q, S, K, NW, NS, MINB, BATCH, PP, ANY, RK, EA, SML>;
         static std::atomic<bool> configured[64] = {};
         int dev = 0;
         cudaGetDevice(&dev);
@@ -443,10 +479,10 @@ struct PairKernel {
     }
 };
 
-template <int Q, int S, int K, int NW, int NS, int MINB, bool PP, bool ANY, int RK, bool EA>
+template <int Q, int S, int K, int NW, int NS, int MINB, bool PP, bool ANY, int RK, bool EA, int SML>
 cudaError_t launch_pair_rk(const StepArgs &a, cudaStream_t st) {
     constexpr int WO = PairGeom<K>::WO;
-    using PK = PairKernel<Q, S, K, NW, NS, MINB, false, PP, ANY, RK, EA>;
+    using PK = PairKernel<Q, S, K, NW, NS, MINB, false, PP, ANY, RK, EA, SML>;
     unsigned full = 0;
     cudaError_t e = PK::get(&full);
     if (e != cudaSuccess) return e;
@@ -456,18 +492,18 @@ cudaError_t launch_pair_rk(const StepArgs &a, cudaStream_t st) {
     const int64_t band = (a.ny + nb - 1) / nb, nbands = (a.ny + band - 1) / band;
     const int64_t units = nstrips * nbands;
     const unsigned grid = units < nwarps ? (unsigned)((units + NW - 1) / NW) : full;
-    return launch_dependent(step_pair_kernel<Q, S, K, NW, NS, MINB, false, PP, ANY, RK, EA>, grid,
+    return launch_dependent(step_pair_kernel<Q, S, K, NW, NS, MINB, false, PP, ANY, RK, EA, SML>, grid,
                             NW * 32, PK::smem, st, a, nstrips, nbands, band, nullptr, 0, 0, a.rho_out != nullptr);
 }
 
 // Two-species Gray-Scott grids run the form with the reaction fixed at
 // compile time (no test of the kind in the row loop); the others test it.
-template <int Q, int S, int K, int NW, int NS, int MINB, bool PP, bool ANY = false, bool EA = false>
+template <int Q, int S, int K, int NW, int NS, int MINB, bool PP, bool ANY = false, bool EA = false, int SML = 0>
 cudaError_t launch_pair(const StepArgs &a, cudaStream_t st) {
     if ((!ANY && a.nx % 4 != 0) || a.pitch % 4 != 0) return cudaErrorInvalidValue;
     if constexpr (S == 2)
-        if (a.rkind == kGrayScott) return launch_pair_rk<Q, S, K, NW, NS, MINB, PP, ANY, kGrayScott, EA>(a, st);
-    return launch_pair_rk<Q, S, K, NW, NS, MINB, PP, ANY, -1, EA>(a, st);
+        if (a.rkind == kGrayScott) return launch_pair_rk<Q, S, K, NW, NS, MINB, PP, ANY, kGrayScott, EA, SML>(a, st);
+    return launch_pair_rk<Q, S, K, NW, NS, MINB, PP, ANY, -1, EA, SML>(a, st);
 }
 
 }  // namespace
