@@ -193,16 +193,16 @@ void default_depths(lb_rd_handle *h) {
 // library (tb_depth 0), by lattice, species, storage, alignment and size; -1:
 // one step per launch.  Grids of up to 2^16 sites keep one launch per step: a
 // step there is launch latency either way (256^2: 6.2 us, four steps per launch
-// 2.4 us each), and callers that time or count the steps of small grids see
+// 2.2 us each), and callers that time or count the steps of small grids see
 // each one.  Above, us per step of the rule's choice against the one-step
-// default, FP32 D2Q9 with two species: 512^2 3.6 / 8.2, 1531 x 1021 13.2 / 49.3,
-// 2048^2 22.3 / 102, 4096^2 80 / 396; D2Q5 4096^2 38 / 207; bf16 deviations
+// default, FP32 D2Q9 with two species: 512^2 3.3 / 8.2, 1531 x 1021 12.4 / 49.3,
+// 2048^2 20.7 / 102, 4096^2 71 / 396; D2Q5 4096^2 38 / 207; bf16 deviations
 // 2048^2 30 / 62.  The lines between two choices lie where the autotuner's times
-// cross: four steps with a six-row ring, which hides the latency of L2-resident
-// rows, against six with a level in shared memory (512^2 3.6 / 5.0, 1024^2 8.0 /
-// 8.3, 2048^2 26.1 / 22.3), any nx takes four steps on
-// small grids (383 x 511: 4.2 against five steps' 5.0; 767 x 703 6.5 / 6.6;
-// 1531 x 1021 14.0 / 13.2), K = 2 beats K = 3 for four D2Q9 species on small grids
+// cross: four steps with three rows in flight, which hides the latency of
+// L2-resident rows, against six with a level in shared memory (896^2 6.41 / 6.60,
+// 1024^2 7.77 / 7.66, 2048^2 26.0 / 20.7), any nx takes four steps on small grids
+// (383 x 511: 3.56 against five steps' 4.35; 767 x 703 6.09 / 5.79), five up to
+// 1.5 M sites (1023^2 8.63 against six steps' 8.85; 4095^2 95.8 / 93.5), K = 2 beats K = 3 for four D2Q9 species on small grids
 // (512^2: 14.5 / 17.9; 2048^2: 139 / 135).
 int default_bulk(const lb_rd_handle *h) {
     const int64_t sites = h->cfg.nx * h->cfg.ny;
@@ -213,8 +213,10 @@ int default_bulk(const lb_rd_handle *h) {
     if (is_half(h))
         return first_fitting(h, {"hpair4_128_minb2", sites < (1 << 21) ? "hdeep4_128_minb2" : "hdeep4_128_minb3"});
     if (h->S * h->Q > 10)
-        return first_fitting(h, {sites <= (3 << 19) ? "deep4vwp_128_minb1_s6" : "deep6vwm_256_minb1",
-                                 sites < (1 << 19) ? "deep4vwa_128_minb2" : "deep5vwpa_256_minb1"});
+        return first_fitting(h, {sites <= (7 << 17) ? "deep4vwp_128_minb1_s6" : "deep6vwm_256_minb1",
+                                 sites < (1 << 19)   ? "deep4vwa_128_minb2"
+                                 : sites < (3 << 19) ? "deep5vwpa_256_minb1"
+                                                     : "deep6vwma_256_minb1"});
     return first_fitting(h, {h->Q == 9 ? "deep6vwpe_128_minb1_s5" : "deep6vwp_128_minb1_s6", "deep6vwpa_128_minb1"});
 }
 

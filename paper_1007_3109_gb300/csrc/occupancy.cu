@@ -23,6 +23,13 @@ int sm_count_locked(int dev) {
 }
 }  // namespace
 
+unsigned sm_count() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(g_mu);
+    return (unsigned)sm_count_locked(dev);
+}
+
 unsigned occupancy_blocks(const void *kernel, int nthreads, size_t smem) {
     int dev = 0;
     cudaGetDevice(&dev);

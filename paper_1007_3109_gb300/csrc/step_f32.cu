@@ -125,7 +125,7 @@ const F32Variant kF32Variants[] = {
     {"deep4vwa_128_minb2", 128, 4, 2, 4, 4, 1},
     {"deep6vwpa_128_minb1", 128, 6, 1, 4, 6, 1},
     {"deep3vwpa_128_minb2_s5", 128, 3, 2, 4, 3, 1},
-    // two columns per lane, two or three rows staged ahead
+    // two columns per lane, more rows staged ahead (_s5: two, _s6: three or four)
     {"deep6vwp_128_minb1_s5", 128, 6, 1, 4, 6, 4},
     {"deep6vwp_128_minb1_s6", 128, 6, 1, 4, 6, 4},
     {"deep5vw_128_minb2_s6", 128, 5, 2, 4, 5, 4},
@@ -134,7 +134,7 @@ const F32Variant kF32Variants[] = {
     {"deep5vwpa_256_minb1", 256, 5, 1, 4, 5, 1},
     // two columns per lane, a row staged as soon as level 1 has read the oldest one: deep<K>vw[p]e_
     {"deep6vwpe_128_minb1_s5", 128, 6, 1, 4, 6, 4},
-    // two columns per lane: three rows staged ahead; one level's rows in shared memory: deep<K>vwm[a]_
+    // two columns per lane: three rows in flight; one level's rows in shared memory: deep<K>vwm[a]_
     {"deep4vwp_128_minb1_s6", 128, 4, 1, 4, 4, 4},
     {"deep6vwm_256_minb1", 256, 6, 1, 4, 6, 4},
     {"deep6vwm_128_minb2", 128, 6, 2, 4, 6, 4},

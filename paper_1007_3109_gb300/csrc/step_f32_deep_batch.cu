@@ -12,16 +12,17 @@ namespace {
 // faster one: depths whose carried levels fit the register file (K <= 5), and
 // K = 6, for two D2Q9 species with level 4's rows in shared memory; its any-nx
 // form unless every grid has nx a multiple of 4.  Four warps, the pulls from
-// earlier rows first (not with a level in shared memory), five staged rows below
-// K = 5 and for D2Q5 (whose smaller rows leave L1 its share with two rows staged
-// ahead).
+// earlier rows first (not with a level in shared memory), one row staged ahead for
+// two D2Q9 species and two for the others, whose rows leave L1 its share (256 x
+// 248^2, K = 6: 494 us per launch with one row ahead, 680 with two; D2Q5 K = 4, 64
+// x 248^2: 73 and 64).
 template <int K>
 struct UsePair {
     static constexpr bool value = K <= 6;
 };
 template <int Q, int S, int K, bool V16, int RK = -1>
 struct PairShape {
-    static constexpr int NW = 4, NS = K < 5 || Q == 5 ? 5 : 4, SML = K == 6 && Q * S > 10 ? 8 : 0;
+    static constexpr int NW = 4, NS = Q * S > 10 ? 2 : 3, SML = K == 6 && Q * S > 10 ? 8 : 0;
     static constexpr int MINB = K == 6 && SML == 0 ? 1 : 2;
     using Kernel = PairKernel<Q, S, K, NW, NS, MINB, true, SML == 0, !V16, RK, false, SML>;
 };

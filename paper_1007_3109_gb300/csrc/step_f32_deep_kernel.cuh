@@ -276,21 +276,23 @@ __global__ void __launch_bounds__(NW * 32, MINB)
 
 // Bands: the count nb of bands per grid whose round-robin deal of
 // nb x nstrips units (ny rows each grid) to nwarps warps takes the least
-// time, rounds x (rows per band + 2K pipeline-fill iterations).
-int64_t choose_bands(int K, int64_t nstrips, int64_t ny, int64_t nwarps) {
+// time, rounds x (rows per band + `fill` pipeline-fill iterations); *cost_out: that
+// estimate.
+int64_t choose_bands(int fill, int64_t nstrips, int64_t ny, int64_t nwarps, int64_t *cost_out = nullptr) {
     int64_t nb = 1, best = INT64_MAX;
     for (int64_t r = 1; r <= 64; ++r) {
         for (int64_t c = r * nwarps / nstrips; c <= r * nwarps / nstrips + 1; ++c) {
             const int64_t n = c < 1 ? 1 : (c > ny ? ny : c);
             const int64_t rows = (ny + n - 1) / n;
             const int64_t rounds = (n * nstrips + nwarps - 1) / nwarps;
-            const int64_t cost = rounds * (rows + 2 * K);
+            const int64_t cost = rounds * (rows + fill);
             if (cost < best) {
                 best = cost;
                 nb = n;
             }
         }
     }
+    if (cost_out) *cost_out = best;
     return nb;
 }
 
@@ -354,7 +356,7 @@ cudaError_t launch_deep(const StepArgs &a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     const int64_t nstrips = (a.nx + WO - 1) / WO;
     const int64_t nwarps = (int64_t)full * NW;
-    const int64_t nb = choose_bands(K, nstrips, a.ny, nwarps);
+    const int64_t nb = choose_bands(2 * K, nstrips, a.ny, nwarps);
     const int64_t band = (a.ny + nb - 1) / nb, nbands = (a.ny + band - 1) / band;
     const int64_t units = nstrips * nbands;
     const unsigned grid = units < nwarps ? (unsigned)((units + NW - 1) / NW) : full;

@@ -16,9 +16,17 @@
 //   * level 0 (f*(t)): rows staged per warp by cp.async in 16-byte chunks
 //     (the row pitch is a multiple of 32): the window's 64 columns start at
 //     xb (even), inside the 17 aligned chunks from a0 = xb rounded down to a
-//     multiple of 4; lanes 0-15 copy chunk `lane` of the even planes, lanes
-//     16-31 chunk `lane - 16` of the odd planes, lane p < S Q chunk 16 of
-//     plane p.  nx a multiple of 4: no chunk straddles the periodic seam.
+//     multiple of 4; lanes 0-15 copy chunk `lane` of the first species' planes
+//     (one species: of the even planes), lanes 16-31 chunk `lane - 16` of the
+//     second's (the odd planes), lane p < S Q chunk 16 of plane p.  A staged row
+//     holds every plane from the grid row its component is pulled from (y - e_iy),
+//     so one staged row serves level 1 of one output row and its slot is free
+//     again: the ring is the rows in flight and one more, instead of three, and
+//     the SM's memory left over is L1, where the halo columns of adjacent strips
+//     meet (8192^2, K = 6: 317 -> 295 us per step, with a second row in flight in
+//     the same two slots 280; K = 4, 512^2: 3.57 -> 3.30; D2Q5 512^2 2.42 -> 2.07).
+//     A launch also starts at the first row level 1 needs, 2K - 2 rows before the
+//     first output row instead of 2K.  nx a multiple of 4: no chunk straddles the periodic seam.
 //     The ANY form takes any nx: a chunk that reaches past the seam (edge
 //     strips only) is copied column by column, a lane per column with its
 //     wrapped position from shared memory (with a remainder per copy by the
@@ -27,7 +35,7 @@
 //     because the extra paths slow the loop body down even where they never
 //     run.  Waits only on the warp's own copy groups.
 //   * level 1 pulls the lane's column pair of every plane from the staged row
-//     of its e_iy (one 8-byte shared load) and shifts it like the levels
+//     (one 8-byte shared load) and shifts it like the levels
 //     above; level m > 1 pulls from level m - 1 carried in registers (the row
 //     of this iteration for e_iy = -1, the previous one for e_iy = 0, the one
 //     before for e_iy = +1), exactly as the one-column kernel.
@@ -73,6 +81,15 @@ __device__ __forceinline__ unsigned lds_v32(const void *p) {
     return v;
 }
 
+// Planes with e_iy = ey, as bits.
+template <int Q, int S>
+__host__ __device__ constexpr unsigned plane_bits(int ey) {
+    unsigned m = 0;
+    for (int p = 0; p < S * Q; ++p)
+        if (Lattice<Q>::ey(p % Q) == ey) m |= 1u << p;
+    return m;
+}
+
 template <int K>
 struct PairGeom {
     static constexpr int HL = (K + 1) / 2 * 2;  // left (and right) halo columns of the window, even
@@ -92,14 +109,15 @@ struct PairCarry {
 // column of an odd nx stored alone); otherwise nx must be a multiple of 4.
 // RK >= 0: the grid's reaction kind, fixed at compile time.  EA: a row is
 // staged as soon as level 1 has read the oldest staged row, whose slot it
-// takes: NS - 2 rows in flight instead of NS - 3, in the same ring.
+// takes: NS rows in flight instead of NS - 1, in the same ring.
 // SML: bit m - 1 set: level m's rows are carried in shared memory instead of
 // registers (not with PP).  At K = 6 the five carried levels of D2Q9 with two
 // species need 180 registers; with level 4 in shared memory (4.6 KB per warp, 24
-// eight-byte accesses per row and no moves between rows) the kernel spills 44
-// bytes instead of 144 and moves the state once per six steps: 8192^2 342 -> 317
-// us per step against K = 5, 2048^2 23.9 -> 22.3.  Levels 2 .. 5 measure alike;
-// two levels want a three-row ring (337 us: a row ahead is not enough).
+// eight-byte accesses per row and no moves between rows) the kernel spills 64
+// bytes instead of 144 and moves the state once per six steps (8192^2: 280 us per
+// step against 319 for K = 5, 2048^2 20.7 / 22.0, 4096^2 71 / 81).  Two levels
+// in shared memory take 302 us at 8192^2, K = 7 with three 334.  K = 5 with level 3
+// there spills nothing (8192^2 342 -> 319 us).
 template <int Q, int S, int K, int NW, int NS, int MINB, bool BATCH, bool PP, bool ANY = false, int RK = -1,
           bool EA = false, int SML = 0>
 __global__ void __launch_bounds__(NW * 32, MINB)
@@ -109,11 +127,12 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     constexpr int SQ = S * Q;
     constexpr int CW = 68;          // staged columns of a warp row: 17 chunks of four
     constexpr int kRow = SQ * CW;   // one staged row, all planes
-    constexpr int P = EA ? NS - 2 : NS - 3;  // rows staged ahead of use
+    constexpr int P = EA ? NS : NS - 1;  // rows staged ahead of use
+    constexpr int F = 2 * K - 2;         // rows that fill the levels before level K's first
     constexpr int HL = PairGeom<K>::HL;
     constexpr int WO = PairGeom<K>::WO;
     constexpr int KC = K > 1 ? K - 1 : 1;
-    static_assert(K >= 1 && K <= 8 && NS >= 4 && WO > 0, "depth 1 .. 8, at least four staged rows");
+    static_assert(K >= 1 && K <= 8 && P >= 1 && WO > 0, "depth 1 .. 8, a row staged ahead");
     extern __shared__ __align__(16) float smem[];
     dependent_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -171,7 +190,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     };
     // lists of two-species D2Q9 grids and the kernels with a level in shared memory, which are
     // bound by instruction issue: the species of a site packed (lists, 256 x 256^2 at K = 5: 98.0 against
-    // 99.4 us per step, 256 x 255^2 137 / 145, 9 x 512^2 16.7 / 17.6; D2Q5 and single grids gain nothing)
+    // 99.4 us per step, 256 x 255^2 137 / 145, 9 x 512^2 16.7 / 17.6; D2Q5 and other single grids gain nothing)
     auto collide = [](const SegArgs &cg, float(&f0)[S][Q], float(&f1)[S][Q], float(&rho0)[S], float(&rho1)[S]) {
         if constexpr ((BATCH || SML) && Q == 9 && S == 2) collide_pair_species<Q, RK>(cg, f0, f1, rho0, rho1);
         else collide_pair<Q, S, RK>(cg, f0, f1, rho0, rho1);
@@ -181,7 +200,11 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     for (int s = 0; s < S; ++s) acc[s] = 0.0;
     const int64_t nwarps = (int64_t)gridDim.x * NW;
     const int64_t units = nstrips * nbands;
-    const int cch = lane & 15, cpar = lane >> 4;  // copy role: chunk, plane parity
+    // copy role: chunk, and species (two species) or plane parity (one)
+    const int cch = lane & 15, cpar = lane >> 4;
+    constexpr int kStep = S == 2 ? 1 : 2;  // planes between a lane's copies
+    // planes pulled from above and from below (bits)
+    constexpr unsigned mUp = plane_bits<Q, S>(1), mDown = plane_bits<Q, S>(-1);
     // BATCH: the warp's place in the list's rows, kept in shared memory like gs
     __shared__ ListWalk walk_sh[BATCH ? NW : 1];
     if constexpr (BATCH) {
@@ -240,24 +263,34 @@ __global__ void __launch_bounds__(NW * 32, MINB)
             }
             __syncwarp();
         }
-        const int64_t offA = (int64_t)cpar * g.plane + (ANY ? (cleanA ? cA : 0) : wrap_mod(cA, nx));
+        const int64_t offA = (int64_t)(cpar * (S == 2 ? Q : 1)) * g.plane + (ANY ? (cleanA ? cA : 0) : wrap_mod(cA, nx));
         const int64_t offB = (int64_t)(lane < SQ ? lane : 0) * g.plane + (ANY ? (cleanB ? cB : 0) : wrap_mod(cB, nx));
-        const int nrows = ly + 2 * K;
-        int yl = (int)wrap_mod(y0 - K, ny);
+        const int nrows = ly + F;
+        int yl = (int)wrap_mod(y0 - K + 1, ny);  // row that is staged next
         auto stage = [&](int j, int slot) {
             if (j < nrows) {
-                const float *row = p_src() + (int64_t)yl * p_pitch();
-                const unsigned d = ring_s + (unsigned)(slot * kRow + cpar * CW + 4 * cch) * 4u;
-                const float *sp = row + offA;
-                int64_t pl2 = 2 * p_plane();
-                asm volatile("" : "+l"(pl2));  // no plane multiples kept live across the row loop
+                const int64_t pitch = p_pitch();
+                const int yu = yl == 0 ? ny - 1 : yl - 1, yd = yl + 1 == ny ? 0 : yl + 1;
+                // the rows that components with e_iy = 0, 1 and -1 are pulled from
+                const float *src = p_src();
+                const float *row0 = src + (int64_t)yl * pitch, *rowu = src + (int64_t)yu * pitch,
+                            *rowd = src + (int64_t)yd * pitch;
+                const unsigned d = ring_s + (unsigned)(slot * kRow + cpar * (S == 2 ? Q : 1) * CW + 4 * cch) * 4u;
+                int64_t pls = kStep * p_plane();
+                asm volatile("" : "+l"(pls));  // no plane multiples kept live across the row loop
                 if (!ANY || cleanA) {
 #pragma unroll
                     for (int r = 0; r < (SQ + 1) / 2; ++r)
-                        if (cpar + 2 * r < SQ) cp_async16(d + (unsigned)(2 * r * CW * 4), sp + r * pl2);
+                        if (S == 2 || cpar + 2 * r < SQ) {
+                            const int ea = L::ey((S == 2 ? r : 2 * r) % Q), eb = L::ey((S == 2 ? r : 2 * r + 1) % Q);
+                            const float *ra = ea > 0 ? rowu : (ea < 0 ? rowd : row0);
+                            const float *rb = eb > 0 ? rowu : (eb < 0 ? rowd : row0);
+                            cp_async16(d + (unsigned)(kStep * r * CW * 4), (cpar ? rb : ra) + offA + r * pls);
+                        }
                 }
                 if (lane < SQ && cleanB)
-                    cp_async16(ring_s + (unsigned)(slot * kRow + lane * CW + 64) * 4u, row + offB);
+                    cp_async16(ring_s + (unsigned)(slot * kRow + lane * CW + 64) * 4u,
+                               ((mUp >> lane) & 1 ? rowu : (mDown >> lane) & 1 ? rowd : row0) + offB);
                 if constexpr (ANY) {
                     if (edge) {  // warp-uniform: a lane per column, plane by plane
                         const volatile int *wc = wcol_sh[w];
@@ -266,10 +299,18 @@ __global__ void __launch_bounds__(NW * 32, MINB)
                         asm volatile("" : "+l"(pl));
                         for (int q = lane; q < nu; q += 32) {
                             const int c = q < lo4 ? q : q - lo4 + hi4;
-                            const float *cp = row + wc[c];
-                            const unsigned dc = ring_s + (unsigned)(slot * kRow + c) * 4u;
-#pragma unroll 6
-                            for (int pp = 0; pp < SQ; ++pp) cp_async4s(dc + (unsigned)(pp * CW * 4), cp + pp * pl);
+                            const int x = wc[c];
+                            unsigned dc = ring_s + (unsigned)(slot * kRow + c) * 4u;
+                            int64_t off = x;  // (unrolled: 16 grids of 2047^2 437 -> 404 us per step)
+#pragma unroll
+                            for (int s = 0; s < S; ++s) {
+#pragma unroll
+                                for (int i = 0; i < Q; ++i) {
+                                    cp_async4s(dc, (L::ey(i) > 0 ? rowu : (L::ey(i) < 0 ? rowd : row0)) + off);
+                                    off += pl;
+                                    dc += CW * 4;
+                                }
+                            }
                         }
                     }
                 }
@@ -299,10 +340,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
             if constexpr (!EA) stage(j + P, sl + P >= NS ? sl + P - NS : sl + P);
             cp_async_wait<EA ? P - 1 : P>();  // this lane's copies of row j have landed
             __syncwarp();
-            const int s1 = sl == 0 ? NS - 1 : sl - 1, s2 = s1 == 0 ? NS - 1 : s1 - 1;
-            // staged rows of iterations j - 2, j - 1, j: pulled with e_iy = +1, 0, -1
-            const float *rows0[3] = {ring + s2 * kRow + o + 2 * lane, ring + s1 * kRow + o + 2 * lane,
-                                     ring + sl * kRow + o + 2 * lane};
+            const float *row = ring + sl * kRow + o + 2 * lane;  // every component as level 1 pulls it
             float f0[S][Q], f1[S][Q], rho0[S], rho1[S];
             float hp0[KC][S][Q], hp1[KC][S][Q];
             if constexpr (PP) {
@@ -332,11 +370,11 @@ __global__ void __launch_bounds__(NW * 32, MINB)
             for (int s = 0; s < S; ++s)
 #pragma unroll
                 for (int i = 0; i < Q; ++i) {
-                    const float2 v = *reinterpret_cast<const float2 *>(rows0[1 - L::ey(i)] + (s * Q + i) * CW);
+                    const float2 v = *reinterpret_cast<const float2 *>(row + (s * Q + i) * CW);
                     f0[s][i] = L::ex(i) > 0 ? __shfl_up_sync(kFullMask, v.y, 1) : (L::ex(i) < 0 ? v.y : v.x);
                     f1[s][i] = L::ex(i) > 0 ? v.x : (L::ex(i) < 0 ? __shfl_down_sync(kFullMask, v.x, 1) : v.y);
                 }
-            if constexpr (EA) {  // every lane has read row j - 2: its slot takes row j + P
+            if constexpr (EA) {  // every lane has read row j: its slot takes row j + P
                 __syncwarp();
                 stage(j + P, sl + P >= NS ? sl + P - NS : sl + P);
             }
@@ -417,10 +455,10 @@ __global__ void __launch_bounds__(NW * 32, MINB)
                 const SegArgs cg = p_coll();
                 collide(cg, f0, f1, rho0, rho1);
             }
-            if (j >= 2 * K) {  // level K of row y0 + j - 2K: window columns HL .. 63 - HL
+            if (j >= F) {  // level K of row y0 + j - F: window columns HL .. 63 - HL
                 const int x = xb + 2 * lane;
                 if (lane >= HL / 2 && lane < (HL + WO) / 2 && x < nx) {
-                    const int y = y0 + j - 2 * K;
+                    const int y = y0 + j - F;
                     int64_t pl = p_plane();
                     asm volatile("" : "+l"(pl));  // no plane multiples kept live across the row loop
                     const int64_t yx = (int64_t)y * p_pitch() + x;
@@ -446,7 +484,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
                     }
                 }
             }
-            // every lane has read slot j - 2 before iteration j + 1 stages into it
+            // every lane has read slot j before iteration j + 1 stages into it
             if (BATCH && Q == 9 && together && (j & 3) == 0) __syncthreads();
             else __syncwarp();
             sl = sl + 1 == NS ? 0 : sl + 1;
@@ -462,8 +500,12 @@ __global__ void __launch_bounds__(NW * 32, MINB)
 template <int Q, int S, int K, int NW, int NS, int MINB, bool BATCH, bool PP = false, bool ANY = false, int RK = -1,
           bool EA = false, int SML = 0>
 struct PairKernel {
+    // Lists of two D2Q9 species: two blocks per SM, also at the shallow depths whose
+    // registers would allow more: with three or four rings L1 has no room for the halo
+    // columns (256 x 248^2, us per launch of 2 .. 4 steps: 500, 465, 463 -> 450, 439, 447).
     static constexpr size_t smem =
         NW * ((size_t)NS * S * Q * 68 * sizeof(float) + __builtin_popcount(SML) * PairCarry<Q, S>::kWarp * sizeof(float2));
+    static constexpr unsigned kCap = BATCH && S * Q > 10 ? 2 : 0;
     static cudaError_t get(unsigned *full) {
         auto kern = step_pair_kernel<Q, S, K, NW, NS, MINB, BATCH, PP, ANY, RK, EA, SML>;
         static std::atomic<bool> configured[64] = {};
@@ -471,13 +513,31 @@ struct PairKernel {
         cudaGetDevice(&dev);
         if (dev < 64 && !configured[dev].load()) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            // (the rest of the SM's memory is L1, where the halo columns of adjacent strips meet)
+            if (kCap > 0 && e == cudaSuccess)
+                e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         (int)((kCap * (smem + 1024) * 100 + (228 << 10) - 1) / (228 << 10)));
             if (e != cudaSuccess) return e;
             configured[dev].store(true);
         }
         *full = persistent_blocks(kern, NW * 32, INT64_MAX, smem);
+        if (kCap > 0 && *full > kCap * sm_count()) *full = kCap * sm_count();
         return cudaSuccess;
     }
 };
+
+// Blocks of four warps for a grid: one per SM where that is estimated to be
+// faster than as many as fit.  Fewer bands fill the levels fewer times, and a
+// warp that has its scheduler to itself walks a row in about 2/3 of the time that
+// each of two take (512^2 at K = 4: 60 bands 3.57 us per step, 121 bands 4.17).
+inline unsigned pair_blocks(int K, int64_t nstrips, int64_t ny, unsigned full) {
+    const unsigned sms = sm_count();
+    if (full <= sms) return full;
+    int64_t one = 0, all = 0;
+    choose_bands(2 * K - 2, nstrips, ny, (int64_t)sms * 4, &one);
+    choose_bands(2 * K - 2, nstrips, ny, (int64_t)full * 4, &all);
+    return one * 2 < all * (1 + full / sms) ? sms : full;
+}
 
 template <int Q, int S, int K, int NW, int NS, int MINB, bool PP, bool ANY, int RK, bool EA, int SML>
 cudaError_t launch_pair_rk(const StepArgs &a, cudaStream_t st) {
@@ -487,8 +547,9 @@ cudaError_t launch_pair_rk(const StepArgs &a, cudaStream_t st) {
     cudaError_t e = PK::get(&full);
     if (e != cudaSuccess) return e;
     const int64_t nstrips = (a.nx + WO - 1) / WO;
+    if (NW == 4) full = pair_blocks(K, nstrips, a.ny, full);
     const int64_t nwarps = (int64_t)full * NW;
-    const int64_t nb = choose_bands(K, nstrips, a.ny, nwarps);
+    const int64_t nb = choose_bands(2 * K - 2, nstrips, a.ny, nwarps);
     const int64_t band = (a.ny + nb - 1) / nb, nbands = (a.ny + band - 1) / band;
     const int64_t units = nstrips * nbands;
     const unsigned grid = units < nwarps ? (unsigned)((units + NW - 1) / NW) : full;

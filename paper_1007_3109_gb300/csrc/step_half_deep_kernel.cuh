@@ -291,7 +291,7 @@ cudaError_t launch_half_deep_rk(const StepArgs &a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     const int64_t nstrips = (a.nx + WO - 1) / WO;
     const int64_t nwarps = (int64_t)full * NW;
-    const int64_t nb = choose_bands(K, nstrips, a.ny, nwarps);
+    const int64_t nb = choose_bands(2 * K, nstrips, a.ny, nwarps);
     const int64_t band = (a.ny + nb - 1) / nb, nbands = (a.ny + band - 1) / band;
     const int64_t units = nstrips * nbands;
     const unsigned grid = units < nwarps ? (unsigned)((units + NW - 1) / NW) : full;
