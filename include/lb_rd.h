@@ -312,7 +312,8 @@ LB_RD_API int lb_rd_batch_init(lb_rd_batch *b, int32_t idx, const double *rho0, 
  * launch also writes each instance's densities: with depth-K launches
  * (lb_rd_batch_set_steps_per_launch) the call runs nsteps / K launches of K
  * steps and one launch of the nsteps % K steps left (a single step if one is
- * left), otherwise its last step is a single step. */
+ * left; FP32: the last full launch and those steps as two of nearly equal
+ * depth), otherwise its last step is a single step. */
 LB_RD_API int lb_rd_batch_step(lb_rd_batch *b, int64_t nsteps);
 
 /* Steps per captured CUDA graph (an even number >= 2), or 0 to launch every
@@ -349,11 +350,9 @@ LB_RD_API int lb_rd_batch_get_time(const lb_rd_batch *b, int64_t *t, int64_t *la
  * Resident requests advance together, steps_per_tick steps at a time (fewer
  * when a request finishes sooner), by launches of the batched kernels over
  * all of them: for FP32 and 16-bit deviation requests with two state copies,
- * tick / K launches of the depth-K kernel (K as a batch of them would take by
- * default) and one launch of the
- * tick % K
- * steps left (a single step if one is left), otherwise one launch per step;
- * the last launch of a tick also writes the densities.  Requests that arrive
+ * tick / K launches of the depth-K kernel (K at most what a batch of them would
+ * take by default) and one launch of the tick % K steps left (a single step if
+ * one is left), otherwise one launch per step; the last launch of a tick also writes the densities.  Requests that arrive
  * meanwhile are admitted between ticks
  * as slots and memory free up.  A finished request's densities and mass are
  * copied to host memory and its device memory is released.  Each result is

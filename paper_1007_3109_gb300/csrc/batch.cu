@@ -568,11 +568,23 @@ int lb_rd_batch_step(lb_rd_batch *b, int64_t nsteps) {
     if (K >= 2 && !uses_tb2(b)) {
         // depth-K launches; the last launch of the call (K steps, or the r =
         // nsteps % K left over: one depth-r launch, a single step for r = 1)
-        // writes the densities
+        // writes the densities.  FP32: the last full launch and the r steps
+        // left are two launches of nearly equal depth, since a launch of one or
+        // two steps takes about as long as one of four (256 grids of 248^2, us
+        // per launch of 1 .. 6 steps: 424, 450, 439, 447, 471, 493)
         const int64_t q = nsteps / K, r = nsteps % K;
-        int rc = run_multi(b, r == 0 ? q - 1 : q);
+        const bool even = r > 0 && r < K - 1 && q > 0 && !half_batch(b);
+        int rc = run_multi(b, r == 0 || even ? q - 1 : q);
         if (rc) return rc;
-        const int d = r == 0 ? K : (int)r;
+        const int tail = r == 0 ? K : (int)r, d0 = even ? (K + tail + 1) / 2 : 0;
+        if (even) {
+            cudaError_t e = launch_deep(b, d0, b->cur, false);
+            if (e) return cuda_err(e, "batch step kernel");
+            b->cur ^= 1;
+            b->t += d0;
+            b->launches++;
+        }
+        const int d = even ? K + tail - d0 : tail;
         cudaError_t e = d == 1 ? launch_one(b, b->cur, true) : launch_deep(b, d, b->cur, true);
         if (e) return cuda_err(e, "batch step kernel");
         b->cur ^= 1;

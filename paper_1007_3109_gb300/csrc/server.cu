@@ -260,9 +260,8 @@ void run_tick(lb_rd_server *s) {
     }
     // K-step launches: FP32 and 16-bit deviation requests with two state
     // copies run the tick as q = tick / K depth-K launches (FP32:
-    // lbrd::batch_deep_default_k; 16-bit storage: lbrd::batch_half_default_k) and, for the r = tick % K
-    // steps left, one
-    // depth-r launch (r >= 2) or one single step (r = 1); the tick's last
+    // K from lbrd::batch_deep_default_k; 16-bit storage: lbrd::batch_half_default_k)
+    // and, for the r = tick % K steps left, one depth-r launch (r >= 2) or one single step (r = 1); the tick's last
     // launch writes the densities.  Other requests: one launch per step.
     bool any_inplace = false;
     for (Request *r : act) any_inplace = any_inplace || r->cfg.streaming == LB_RD_STREAM_INPLACE;
@@ -272,7 +271,11 @@ void run_tick(lb_rd_server *s) {
     const bool half = s->mode == 1 || s->mode == 2;  // 16-bit deviation storage: its own depth-K kernels
     int64_t sites = 0;
     for (Request *r : act) sites += r->cfg.nx * r->cfg.ny;
-    const int K = half ? lbrd::batch_half_default_k() : lbrd::batch_deep_default_k(s->Q, s->cfg.nspecies, sites);
+    // FP32: as many launches as the default depth Kd takes, of nearly equal depth (a launch
+    // of one or two steps takes about as long as one of four)
+    const int Kd = half ? lbrd::batch_half_default_k() : lbrd::batch_deep_default_k(s->Q, s->cfg.nspecies, sites);
+    const int64_t nl = (tick + Kd - 1) / Kd;
+    const int K = half ? Kd : std::max<int>(2, (int)((tick + nl - 1) / nl));
     const bool deep = (s->mode == 0 || half) && !any_inplace && tick >= 2;
     int64_t n_multi = deep ? tick / K : 0;
     int rem = deep ? (int)(tick % K) : 0;  // steps of the depth-r launch (0: none)
