@@ -45,7 +45,8 @@ __device__ __forceinline__ void weighted(double v, double (&c)[Lattice<Q>::kClas
     c[1] = __dmul_rn(L::template wc<double>(1), v);
     const int hi = __double2hiint(c[1]), lo = __double2loint(c[1]);
     const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
-    const bool zero = ((hi & 0x7fffffff) | lo) == 0;
+    // v itself, not the product: w_1 v rounds to zero for the smallest v whose w_0 v does not
+    const bool zero = ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0;
     // exponents 3 .. 2043: the product and its multiples by 1/4 .. 4 are normal; zero stays zero
     const bool plain = e - 3u <= 2040u || zero;
     const unsigned warp = __activemask();
