@@ -189,10 +189,15 @@ cudaError_t launch_batch_tb2(const TbwItem *items, int n, int64_t total_units, i
 // rho(t + K) of every item to its a.rho_out (the last launch of a call).
 // rk: the reaction kind that every item has (a.rkind), or -1 when they differ
 // (list_reaction_kind); selects a kernel with the kind fixed at compile time.
+struct ListRun {          // consecutive grids of equal shape (list_rows.cuh)
+    int64_t begin, end;  // its rows (past the last run: INT64_MAX)
+    int item, ny;        // its first grid, and their height
+};
 struct DeepItem {
     StepArgs a;
     int64_t unit_begin, nstrips, band;
     int64_t run_strips, next, height;  // two-column kernels: the list's rows (list_rows.cuh)
+    ListRun run;                       // of item k: run number k
     int gs, lockstep;
 };
 // The same over 16-bit deviation storage (K = 2 .. 5; half_kind 0 bf16, 1 fp16;

@@ -32,14 +32,33 @@ namespace {
 // closer to L2 lose a little instead (9 x 512^2, 2.4 M sites: 16.7 -> 17.3).
 constexpr int64_t kLockstepSites = 8 << 20;
 
+// The run of row u, at or after run r: bisection over the runs, which the items
+// hold in order.  Each look is a memory latency that depends on the one before, at
+// the start of every launch (a run's end stands beside its begin: one look for a
+// list of one run).  With a walk from run to run the last workers of 300 grids of
+// seven sizes began 85 us late (D2Q9, one species, 60 steps: 1404 us, with bisection
+// 357; 120 different grids of 64 .. 183 columns, D2Q5: 1446 and 915).  Out of line:
+// inlined, 256 x 256^2 with bf16 deviations took 116.1 us per step instead of 115.0.
+__device__ __noinline__ int list_rows_run(const DeepItem *__restrict__ items, int nitems, int64_t u, int r) {
+    if (u < items[r].run.end) return r;
+    int hi = nitems;
+    while (hi - r > 1) {
+        const int mid = (r + hi) / 2;
+        if (items[mid].run.begin <= u) r = mid;
+        else hi = mid;
+    }
+    return r;
+}
+
 // A cut of the line moved to the end of a strip that is at most `slack` rows
-// away, so that no worker fills the levels for a few rows of a strip.
+// away, so that no worker fills the levels for a few rows of a strip.  r: a run
+// at or before the cut's, which it becomes.
 __device__ __forceinline__ int64_t list_rows_snap(const DeepItem *__restrict__ items, int nitems, int64_t u,
-                                                  int64_t total, int slack, int &run) {
+                                                  int64_t total, int slack, int &r) {
     if (u <= 0 || u >= total) return u;
-    for (int nx = (int)items[run].next; nx < nitems && items[nx].unit_begin <= u; nx = (int)items[run].next) run = nx;
-    const int ny = (int)items[run].a.ny;
-    const int at = (int)((u - items[run].unit_begin) % ny);
+    r = list_rows_run(items, nitems, u, r);
+    const int ny = items[r].run.ny;
+    const int at = (int)((u - items[r].run.begin) % ny);
     return at <= slack ? u - at : (ny - at <= slack ? u + (ny - at) : u);
 }
 
@@ -66,15 +85,16 @@ __device__ __forceinline__ void list_rows_begin(const DeepItem *__restrict__ ite
         walk.u = worker * band;
         walk.u_end = total;
         walk.stride = nworkers * band;
+        if (walk.u < total) walk.run = items[list_rows_run(items, nitems, walk.u, 0)].run.item;
         return;
     }
     walk.stride = 0;
     const int64_t rows = total / nworkers;
     const int slack = rows + 1 < 2 * K ? (int)(rows + 1) / 2 : K;
-    int run = 0;
-    walk.u = list_rows_snap(items, nitems, total * worker / nworkers, total, slack, run);
-    walk.run = run;
-    walk.u_end = list_rows_snap(items, nitems, total * (worker + 1) / nworkers, total, slack, run);
+    int r = 0;
+    walk.u = list_rows_snap(items, nitems, total * worker / nworkers, total, slack, r);
+    walk.run = items[r].run.item;
+    walk.u_end = list_rows_snap(items, nitems, total * (worker + 1) / nworkers, total, slack, r);
 }
 
 // The next segment: rows [y0, y0 + ly) of strip `strip` of grid `item`;
@@ -117,7 +137,7 @@ __device__ __forceinline__ int list_rows_next(const DeepItem *__restrict__ items
 // length of the line.
 inline int64_t plan_list_rows(DeepItem *items, int n, int K, int WO, int NW, int64_t nblocks) {
     int64_t strip_rows = 0, group_rows = 0, planes = 0;
-    int maxny = 1;
+    int maxny = 1, nruns = 0;
     for (int i = 0; i < n;) {
         int j = i + 1;
         while (j < n && items[j].a.nx == items[i].a.nx && items[j].a.ny == items[i].a.ny) ++j;
@@ -131,6 +151,7 @@ inline int64_t plan_list_rows(DeepItem *items, int n, int K, int WO, int NW, int
         strip_rows += total * items[i].a.ny;
         group_rows += (total + NW - 1) / NW * items[i].a.ny;
         if (items[i].a.ny > maxny) maxny = (int)items[i].a.ny;
+        items[nruns++].run.item = i;
         i = j;
     }
     const int gs = group_rows * NW <= 2 * strip_rows ? NW : 1;
@@ -155,7 +176,8 @@ inline int64_t plan_list_rows(DeepItem *items, int n, int K, int WO, int NW, int
         if (lo <= rows / workers + 2 * K) band = lo;
     }
     int64_t at = 0;
-    for (int i = 0; i < n; i = (int)items[i].next) {
+    for (int r = 0; r < nruns; ++r) {
+        const int i = items[r].run.item;
         // a group's place on the line: its rows, or its bands' rows rounded up
         const int64_t height = band > 0 ? (items[i].a.ny + band - 1) / band * band : items[i].a.ny;
         for (int k = i; k < items[i].next; ++k) {
@@ -165,8 +187,11 @@ inline int64_t plan_list_rows(DeepItem *items, int n, int K, int WO, int NW, int
             items[k].height = height;
             items[k].unit_begin = at;
         }
+        const int64_t begin = at;
         at += (items[i].run_strips + gs - 1) / gs * height;
+        items[r].run = {begin, at, i, (int)items[i].a.ny};
     }
+    for (int r = nruns; r < n; ++r) items[r].run.begin = INT64_MAX;
     return at;
 }
 
