@@ -262,18 +262,18 @@ __device__ __forceinline__ void block_mass_reduce(double (&acc)[S], double *part
 }
 
 // Programmatic dependent launch: a kernel launched with launch_dependent
-// (lbrd_kernels.h) may start while the kernel before it on the stream is still
-// running, and calls this before its first access to global memory; it returns
-// when that kernel has completed and its writes are visible.  The second
-// instruction lets the kernel after this one start as soon as every block of
-// this one is running.  A step is a chain of dependent launches, and each left
-// the GPU idle for about 3 us (128^2 FP64: 6.6 us per step, 3.6 so).  For kernels
-// that read the state by plain loads, cp.async or bulk copies only: the read-only
-// path (ld.global.nc) wants memory that nobody writes while the kernel is resident.
-__device__ __forceinline__ void dependent_wait() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// (lbrd_kernels.h) is started as soon as the last block of the kernel before it on
+// the stream has ended, and calls this before its first access to global memory;
+// it returns when that kernel has completed and its writes are visible.  A step is
+// a chain of dependent launches, and each left the GPU idle for about 3 us (128^2
+// FP64: 6.2 us per step, 3.6 so).  No kernel lets the next one start earlier
+// (griddepcontrol.launch_dependents): the next one's blocks, waiting, would fill the
+// SMs that this one's leave free and run unevenly spread (FP64, 512 x 160, D2Q5, two
+// species: 14.1 us per step so, 21.4 with that at the start of every block; 512^2
+// 57.7 either way).  For kernels that read the state by plain loads, cp.async or
+// bulk copies only: the read-only path (ld.global.nc) wants memory that nobody
+// writes while the kernel is resident.
+__device__ __forceinline__ void dependent_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __host__ __device__ inline int64_t wrap(int64_t a, int64_t n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
