@@ -239,6 +239,20 @@ cudaError_t plan_deep(lb_rd_batch *b, int K) {
     return e;
 }
 
+// Whether a call's last steps can be launched at depths d0 and d1: their
+// descriptors are planned here, before any of the call's launches.  Not while the
+// stream is captured (planning allocates and copies), nor where the memory for them
+// is lacking: the call then runs full launches and the remainder.
+bool can_split(lb_rd_batch *b, int d0, int d1) {
+    if (b->deep_units[d0] > 0 && b->deep_units[d1] > 0) return true;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const bool ok = cudaStreamIsCapturing(b->stream, &capture) == cudaSuccess &&
+                    capture == cudaStreamCaptureStatusNone && plan_deep(b, d0) == cudaSuccess &&
+                    plan_deep(b, d1) == cudaSuccess;
+    if (!ok) cudaGetLastError();  // clear a non-sticky error of the attempt
+    return ok;
+}
+
 // One depth-K launch of K steps from buffer parity `parity`; emit: it also
 // writes every instance's densities.
 cudaError_t launch_deep(lb_rd_batch *b, int K, int parity, bool emit) {
@@ -573,10 +587,10 @@ int lb_rd_batch_step(lb_rd_batch *b, int64_t nsteps) {
         // two steps takes about as long as one of four (256 grids of 248^2, us
         // per launch of 1 .. 6 steps: 424, 450, 439, 447, 471, 493)
         const int64_t q = nsteps / K, r = nsteps % K;
-        const bool even = r > 0 && r < K - 1 && q > 0 && !half_batch(b);
+        const int tail = r == 0 ? K : (int)r, d0 = (K + tail + 1) / 2;
+        const bool even = r > 0 && r < K - 1 && q > 0 && !half_batch(b) && can_split(b, d0, K + tail - d0);
         int rc = run_multi(b, r == 0 || even ? q - 1 : q);
         if (rc) return rc;
-        const int tail = r == 0 ? K : (int)r, d0 = even ? (K + tail + 1) / 2 : 0;
         if (even) {
             cudaError_t e = launch_deep(b, d0, b->cur, false);
             if (e) return cuda_err(e, "batch step kernel");
