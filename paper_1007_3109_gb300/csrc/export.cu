@@ -4,6 +4,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "lbrd_kernels.h"
 #include "lb_rd.h"
 
@@ -220,9 +222,10 @@ cudaError_t launch_export(int prec, int Q, int S, const void *state, int64_t nx,
     return cudaGetLastError();
 }
 
+// One per block of the read-out: no more than fit the device, whatever the grid.
 size_t mass_partials_needed(int64_t nx, int64_t ny) {
     int64_t tiles_x = 0;
-    return (size_t)readout_tiles(nx, ny, &tiles_x);
+    return (size_t)std::min<int64_t>(readout_tiles(nx, ny, &tiles_x), max_persistent_blocks());
 }
 
 cudaError_t launch_readout(int prec, int S, const void *rho, int64_t nx, int64_t ny, int64_t pitch, double *out,

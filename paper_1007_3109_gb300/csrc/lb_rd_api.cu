@@ -361,9 +361,8 @@ int lb_rd_check_config(const lb_rd_config *cfg, size_t *bytes) {
         const int64_t pitch = pitch_for(cfg->nx);
         const size_t st = lbrd::state_plane_bytes(cfg->precision, Q, cfg->nspecies, cfg->ny, pitch);
         const size_t rb = (size_t)cfg->nspecies * cfg->ny * pitch * rho_elem(cfg->precision);
-        const size_t np1 = lbrd::max_persistent_blocks(), np2 = lbrd::mass_partials_needed(cfg->nx, cfg->ny);
         const size_t copies = cfg->streaming == LB_RD_STREAM_INPLACE ? 1 : 2;
-        *bytes = copies * st + rb + (np1 > np2 ? np1 : np2) * cfg->nspecies * sizeof(double) +
+        *bytes = copies * st + rb + lbrd::max_persistent_blocks() * cfg->nspecies * sizeof(double) +
                  LB_RD_MAX_SPECIES * sizeof(double) + 2 * sizeof(int);
     }
     return LB_RD_OK;
@@ -410,9 +409,7 @@ int lb_rd_create(const lb_rd_config *cfg, lb_rd_handle **out) {
     h->stream = static_cast<cudaStream_t>(cfg->stream);
     h->state_bytes = lbrd::state_plane_bytes(h->prec, h->Q, h->S, cfg->ny, h->pitch);
     h->rho_bytes = (size_t)h->S * h->plane * rho_elem(h->prec);
-    const size_t nparts = (size_t)lbrd::max_persistent_blocks();
-    const size_t nparts2 = lbrd::mass_partials_needed(cfg->nx, cfg->ny);
-    const size_t parts = (nparts > nparts2 ? nparts : nparts2) * h->S;
+    const size_t parts = (size_t)lbrd::max_persistent_blocks() * h->S;  // a step's or a read-out's, one per block
     cudaError_t err = cudaSuccess;
     if (!err) err = cudaMalloc(&h->buf[0], h->state_bytes);
     if (!err && !h->inplace) err = cudaMalloc(&h->buf[1], h->state_bytes);

@@ -98,7 +98,6 @@ struct lb_rd_server {
     double *partials = nullptr;
     unsigned int *counter = nullptr;
     double *d_mass = nullptr;
-    size_t partials_cap = 0;
     int64_t launches = 0, ticks = 0, finished = 0;
     std::string worker_error;
 };
@@ -172,13 +171,6 @@ int collect_request(lb_rd_server *s, Request *r) {
     double *stage = nullptr;
     cudaError_t e = cudaMallocAsync((void **)&stage, n * sizeof(double), s->stream);
     const int prec = c.precision == LB_RD_FP64 ? LB_RD_FP64 : LB_RD_FP32;  // density cache is float
-    const size_t parts = lbrd::mass_partials_needed(c.nx, c.ny) * 2;
-    if (!e && parts > s->partials_cap) {
-        cudaFreeAsync(s->partials, s->stream);
-        s->partials = nullptr;
-        e = cudaMallocAsync((void **)&s->partials, parts * sizeof(double), s->stream);
-        if (!e) s->partials_cap = parts;
-    }
     if (!e) e = lbrd::launch_readout(prec, c.nspecies, r->rho, c.nx, c.ny, r->pitch, stage, s->partials, s->counter,
                                      s->d_mass, s->stream);
     r->rho_out.resize(n);
@@ -474,8 +466,8 @@ int lb_rd_server_create(const lb_rd_server_config *cfg, lb_rd_server **out) {
         uint64_t keep = cfg->hbm_budget_bytes;
         cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
-    s->partials_cap = lbrd::mass_partials_needed(4096, 4096) * 2;
-    if (!e) e = cudaMalloc(&s->partials, s->partials_cap * sizeof(double));
+    // as many as the read-out of any grid can need
+    if (!e) e = cudaMalloc(&s->partials, lbrd::max_persistent_blocks() * 2 * sizeof(double));
     if (!e) e = cudaMalloc(&s->counter, sizeof(unsigned int));
     if (!e) e = cudaMemset(s->counter, 0, sizeof(unsigned int));
     if (!e) e = cudaMalloc(&s->d_mass, 2 * sizeof(double));
