@@ -188,6 +188,7 @@ int ensure_items(lb_rd_server *s, size_t n) {
     cudaFreeHost(s->h_items);
     s->d_items = nullptr;
     s->h_items = nullptr;
+    s->items_cap = 0;  // until both allocations below have succeeded
     const size_t cap = 3 * std::max<size_t>(n, 64);
     if (cudaMalloc(&s->d_items, cap * sizeof(lbrd::BatchItem)) != cudaSuccess) return LB_RD_ENOMEM;
     if (cudaMallocHost(&s->h_items, cap * sizeof(lbrd::BatchItem)) != cudaSuccess) return LB_RD_ENOMEM;
@@ -202,6 +203,7 @@ int ensure_deep(lb_rd_server *s, size_t n) {
     cudaFreeHost(s->h_deep);
     s->d_deep = nullptr;
     s->h_deep = nullptr;
+    s->deep_cap = 0;
     const size_t cap = 3 * std::max<size_t>(n, 64);
     if (cudaMalloc(&s->d_deep, cap * sizeof(lbrd::DeepItem)) != cudaSuccess) return LB_RD_ENOMEM;
     if (cudaMallocHost(&s->h_deep, cap * sizeof(lbrd::DeepItem)) != cudaSuccess) return LB_RD_ENOMEM;
