@@ -249,7 +249,10 @@ LB_RD_API int lb_rd_launch_count(const lb_rd_handle *h, int64_t *launches);
  * single-step variant and, if faster per step, a multi-step variant, and
  * records the fastest depth-K variant of every depth with its time; the
  * choice is cached per (device, precision, lattice, species, nx, ny) and
- * handles created later with the same shape start from it.  With a K-step
+ * reaction (its kind; a network's number of steps and largest order), and
+ * handles created later with the same shape start from that of their reaction,
+ * else from the last one of the shape (more than two species or a network:
+ * from the choice by size where tb_depth describes one).  With a K-step
  * variant lb_rd_step advances K steps per launch; with a depth-K variant its
  * last r + K min(q, 4) steps (nsteps = q K + r) go in launches of 1 .. K
  * steps, fastest total by the recorded times (untuned: a fixed relative

@@ -99,7 +99,7 @@ struct lb_rd_handle {
 extern "C" const char *lb_rd_handle_variant_name(const lb_rd_handle *h, int32_t variant);
 
 namespace {
-// Autotuner choices per (device, precision, Q, S, nx, ny): single-step
+// Autotuner choices per (device, precision, Q, S, nx, ny) and reaction: single-step
 // variant, multi-step variant (-1 if none is faster) and the fastest depth-K
 // variant with its time per step for every d = 2 .. 8.
 struct TuneEntry {
@@ -107,14 +107,53 @@ struct TuneEntry {
     int depth_variant[9] = {-1, -1, -1, -1, -1, -1, -1, -1, -1};
     double depth_ms[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
 };
+struct ShapeTunes {
+    std::map<int, TuneEntry> by_reaction;
+    int last = 0;  // the reaction tuned last
+};
+using ShapeKey = std::tuple<int, int, int, int, int64_t, int64_t>;
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int64_t, int64_t>, TuneEntry> g_tune_cache;
+std::map<ShapeKey, ShapeTunes> g_tune_cache;
 
-std::tuple<int, int, int, int, int64_t, int64_t> tune_key(const lb_rd_handle *h) {
+ShapeKey shape_key(const lb_rd_handle *h) {
     int dev = 0;
     cudaGetDevice(&dev);
-    return std::make_tuple(dev, h->prec + (h->general ? 16 : 0) + (h->inplace ? 32 : 0), h->Q, h->S, h->cfg.nx,
-                           h->cfg.ny);
+    return ShapeKey(dev, h->prec + (h->general ? 16 : 0) + (h->inplace ? 32 : 0), h->Q, h->S, h->cfg.nx, h->cfg.ny);
+}
+
+// What of a reaction decides the cost of a step: its kind and, for a network, its
+// steps in groups of four and whether it has third powers.
+int tune_reaction(const lb_rd_reaction &r) {
+    if (r.kind != LB_RD_REACTION_MASS_ACTION) return r.kind;
+    bool cubes = false;
+    for (int q = 0; q < r.nreactions; ++q)
+        for (int j = 0; j < LB_RD_MAX_SPECIES; ++j) cubes = cubes || r.order[q][j] > 2;
+    return r.kind + 16 * ((r.nreactions + 3) / 4) + (cubes ? 256 : 0);
+}
+
+int default_bulk(const lb_rd_handle *h);
+
+// The tuned choice a handle starts from (g_tune_mu held), or null: that of its
+// reaction, else the last one of its shape, since the kernels of at most two species
+// cost about the same with any reaction.  Not so the general kernel, whose best depth
+// depends on the network: there the rule by size, where it has a choice, comes before
+// another reaction's (four D2Q9 species at 2048^2, us per step: gdeep3_128_minb2, the
+// fastest without a reaction at 82, takes 152 with ten network steps and 186 with 16,
+// the rule's gdeep3_128_minb3 135 and 171).
+const TuneEntry *find_tune(const lb_rd_handle *h) {
+    auto it = g_tune_cache.find(shape_key(h));
+    if (it == g_tune_cache.end()) return nullptr;
+    auto own = it->second.by_reaction.find(tune_reaction(h->cfg.reaction));
+    if (own != it->second.by_reaction.end()) return &own->second;
+    if (h->general && default_bulk(h) >= 0) return nullptr;
+    return &it->second.by_reaction.at(it->second.last);
+}
+
+void keep_tune(const lb_rd_handle *h, const TuneEntry &t) {
+    std::lock_guard<std::mutex> lock(g_tune_mu);
+    ShapeTunes &s = g_tune_cache[shape_key(h)];
+    s.last = tune_reaction(h->cfg.reaction);
+    s.by_reaction[s.last] = t;
 }
 
 int variant_count(int prec) {
@@ -431,9 +470,8 @@ int lb_rd_create(const lb_rd_config *cfg, lb_rd_handle **out) {
     default_depths(h);
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        auto it = g_tune_cache.find(tune_key(h));
-        if (it != g_tune_cache.end()) {
-            apply_tune(h, it->second);
+        if (const TuneEntry *t = find_tune(h)) {
+            apply_tune(h, *t);
         } else if (cfg->tb_depth == 0) {
             h->tb_variant = default_bulk(h);
             h->by_size = h->tb_variant >= 0;
@@ -823,12 +861,11 @@ int lb_rd_set_variant(lb_rd_handle *h, int32_t variant) {
     if (!h) return fail(LB_RD_EINVAL, "handle is NULL");
     if (variant == -1) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        auto it = g_tune_cache.find(tune_key(h));
         default_depths(h);
         h->variant = 0;
         h->tb_variant = h->cfg.tb_depth == 0 ? default_bulk(h) : -1;
         h->by_size = h->tb_variant >= 0;
-        if (it != g_tune_cache.end()) apply_tune(h, it->second);
+        if (const TuneEntry *t = find_tune(h)) apply_tune(h, *t);
         return LB_RD_OK;
     }
     if (variant < 0 || variant >= handle_variant_count(h))
@@ -906,12 +943,9 @@ static int autotune_inplace(lb_rd_handle *h, int32_t iters, int32_t *best, doubl
     if (e) return cuda_fail(e, "in-place autotune");
     h->variant = bestv >= 0 ? bestv : 0;
     h->tb_variant = -1;
-    {
-        std::lock_guard<std::mutex> lock(g_tune_mu);
-        TuneEntry t;
-        t.variant = h->variant;
-        g_tune_cache[tune_key(h)] = t;
-    }
+    TuneEntry te;
+    te.variant = h->variant;
+    keep_tune(h, te);
     if (best) *best = h->variant;
     return LB_RD_OK;
 }
@@ -983,10 +1017,7 @@ int lb_rd_autotune(lb_rd_handle *h, int32_t iters, int32_t *best, double *times_
     default_depths(h);
     apply_tune(h, te);
     const int arg = h->tb_variant >= 0 ? h->tb_variant : h->variant;
-    {
-        std::lock_guard<std::mutex> lock(g_tune_mu);
-        g_tune_cache[tune_key(h)] = te;
-    }
+    keep_tune(h, te);
     if (best) *best = arg;
     return LB_RD_OK;
 }
