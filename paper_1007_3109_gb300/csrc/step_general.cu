@@ -383,9 +383,10 @@ cudaError_t dispatch_init(int Q, int S, const InitArgs &a, cudaStream_t st) {
 
 }  // namespace
 
+// Programs pick variants by name or index: new ones go to the end.
 const GeneralVariant kGeneralVariants[] = {
     {"general_1site", 1, 1}, {"general_2site", 2, 1}, {"general_4site", 4, 1}, {"general_2site_minb3", 2, 1},
-    {"general_2pass_minb10", 1, 1},
+    {"general_2pass_minb8", 1, 1}, {"general_2pass_minb10", 1, 1},
     // K steps per launch (step_general_deep.cu)
     {"gdeep2_128_minb3", 4, 2}, {"gdeep2_128_minb2", 4, 2}, {"gdeep3_128_minb3", 4, 3}, {"gdeep3_128_minb2", 4, 3},
 };
@@ -398,8 +399,9 @@ cudaError_t launch_step_general(int prec, int Q, int S, const StepArgs &a, cudaS
         case 1: return dispatch_vec<2, 4>(Q, S, a, st);
         case 2: return dispatch_vec<4, 2>(Q, S, a, st);
         case 3: return dispatch_vec<2, 3>(Q, S, a, st);
-        case 4: return dispatch_2pass<10>(Q, S, a, st);
-        case 5: case 6: case 7: case 8: return launch_step_general_deep(variant - 5, Q, S, a, st);
+        case 4: return dispatch_2pass<8>(Q, S, a, st);
+        case 5: return dispatch_2pass<10>(Q, S, a, st);
+        case 6: case 7: case 8: case 9: return launch_step_general_deep(variant - 6, Q, S, a, st);
         default: return cudaErrorInvalidValue;
     }
 }
