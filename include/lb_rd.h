@@ -141,7 +141,11 @@ typedef struct {
     double tau[LB_RD_MAX_SPECIES]; /* relaxation time per species, > 1/2 (D = (tau - 1/2)/3) */
     lb_rd_reaction reaction;
     int32_t precision;       /* lb_rd_precision */
-    int32_t track_mass;      /* nonzero: every step also reduces sum_x rho_s in FP64 */
+    int32_t track_mass;      /* nonzero: step launches also reduce sum_x rho_s (in FP64; FP32 and 16-bit
+                                storage add FP32 partial sums of a thread's sites, grouped by the
+                                launch variant: masses of two variants, and so of a tuned and an
+                                untuned handle, agree to about 1e-9 relative, not bit
+                                for bit) */
     int32_t streaming;       /* lb_rd_streaming */
     void *stream;            /* cudaStream_t for all work; NULL = legacy default stream */
     int32_t tb_depth;        /* time steps per launch (temporal blocking): 0 = the autotuner's cached choice
@@ -194,7 +198,8 @@ LB_RD_API int lb_rd_init(lb_rd_handle *h, const double *rho0, int is_device);
  * steps also writes the densities rho(t), so that no single-step launch is
  * needed to leave them available.  An untuned handle of more than 65536 sites
  * (tb_depth 0) runs a depth-K variant chosen by its size, with the same
- * results; with track_mass its call ends on a single step. */
+ * results; with track_mass its call ends on a single step, whose mass has the
+ * bits of one step per launch. */
 LB_RD_API int lb_rd_step(lb_rd_handle *h, int64_t nsteps);
 
 /* Current time step t of the handle. */
@@ -202,8 +207,8 @@ LB_RD_API int lb_rd_get_time(const lb_rd_handle *h, int64_t *t);
 
 /* Densities rho_s(x, t) = sum_i f_i,s(x, t) at the current time (pre-collision,
  * i.e. after t streams; t = 0 gives sum_i w_i rho0).  rho_out: [S][ny][nx]
- * FP64 or NULL; mass_out: S doubles, sum over all sites of rho_s, reduced in
- * FP64, or NULL.  Synchronises the handle's stream. */
+ * FP64 or NULL; mass_out: S doubles, sum over all sites of rho_s, added in
+ * FP64 (with track_mass after a step: that step's reduction), or NULL.  Synchronises the handle's stream. */
 LB_RD_API int lb_rd_moments(lb_rd_handle *h, double *rho_out, double *mass_out, int is_device);
 
 /* Post-collision distributions f*_i,s(x, t) (the values about to be streamed

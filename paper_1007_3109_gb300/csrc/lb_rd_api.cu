@@ -230,19 +230,21 @@ void default_depths(lb_rd_handle *h) {
 
 // The multi-step variant of an untuned handle that leaves the depth to the
 // library (tb_depth 0), by lattice, species, storage, alignment and size; -1:
-// one step per launch.  Grids of up to 2^16 sites keep one launch per step: a
-// step there is launch latency either way (256^2: 6.2 us, four steps per launch
-// 2.2 us each), and callers that time or count the steps of small grids see
-// each one.  Above, us per step of the rule's choice against the one-step
-// default, FP32 D2Q9 with two species: 512^2 3.3 / 8.2, 1531 x 1021 12.4 / 49.3,
-// 2048^2 20.7 / 102, 4096^2 71 / 396; D2Q5 4096^2 38 / 207; bf16 deviations
-// 2048^2 30 / 62.  The lines between two choices lie where the autotuner's times
-// cross: four steps with three rows in flight, which hides the latency of
-// L2-resident rows, against six with a level in shared memory (896^2 6.41 / 6.60,
-// 1024^2 7.77 / 7.66, 2048^2 26.0 / 20.7), any nx takes four steps on small grids
-// (383 x 511: 3.56 against five steps' 4.35; 767 x 703 6.09 / 5.79), five up to
-// 1.5 M sites (1023^2 8.63 against six steps' 8.85; 4095^2 95.8 / 93.5), K = 2 beats K = 3 for four D2Q9 species on small grids
-// (512^2: 14.5 / 17.9; 2048^2: 139 / 135).
+// one step per launch.  Grids of up to 2^16 sites keep one launch per step, for
+// callers that time or count the steps of small grids: in FP32 that costs them time
+// (256^2: 6.2 us per step against 2.1 with four steps per launch; a tuned handle or
+// a variant of several steps has it), with 16-bit deviations it does not (4.2
+// against 4.5).  Above, us per step of the rule's choice against the one-step
+// default, FP32 D2Q9 with two species: 512^2 3.3 / 8.2, 1531 x 1021 11.8 / 49.6,
+// 2048^2 20.5 / 115, 4096^2 73 / 440; D2Q5 4096^2 39 / 230; bf16 deviations
+// 512^2 5.7 / 8.3, 2048^2 29.8 / 61.6.  The lines between two choices were put where
+// the autotuner's times crossed; now: four steps with three rows in flight, which
+// hides the latency of L2-resident rows, against six with a level in shared memory
+// 896^2 5.87 / 6.49, 1024^2 7.31 / 7.48, 1280^2 10.99 / 9.80, 2048^2 25.0 / 20.5;
+// any nx, four, five and six steps: 383 x 511 3.34 / 4.08 / 4.42, 767 x 703 5.82 /
+// 5.62 / 5.90, 895 x 901 6.82 / 7.70 / 7.61, 1023^2 9.92 / 8.32 / 8.23, 1531 x 1021
+// 12.9 / 11.8 / 11.3, 4095^2 140 / 95 / 85; four D2Q9 species, two and three steps:
+// 512^2 13.3 / 17.0, 1448^2 71.1 / 70.1, 2048^2 138 / 134.
 int default_bulk(const lb_rd_handle *h) {
     const int64_t sites = h->cfg.nx * h->cfg.ny;
     if (sites <= (1 << 16) || h->inplace || h->prec == LB_RD_FP64) return -1;
@@ -605,7 +607,9 @@ int lb_rd_step(lb_rd_handle *h, int64_t nsteps) {
     // from the other copy (ensure_rho).
     // A handle on the size rule with a tracked mass ends on a single step, which
     // reduces the mass (only the last step's can be read): the same masses, bit
-    // for bit, as with one step per launch.
+    // for bit, as with one step per launch of the default variant.  (A handle that
+    // starts from a tuned choice may end on a launch of several steps, whose FP32
+    // partial sums are grouped otherwise.)
     const bool mass_last = h->by_size && h->cfg.track_mass;
     const LaunchPlan plan = plan_launches(h, nsteps, mass_last);
     const int64_t nl = plan.bulk + (int64_t)plan.tail.size();
@@ -837,6 +841,7 @@ int lb_rd_variant_count(int32_t precision, int32_t *count) {
 const char *lb_rd_variant_name(int32_t precision, int32_t variant) {
     if (precision == LB_RD_FP32 && variant >= 0 && variant < lbrd::kF32VariantCount)
         return lbrd::kF32Variants[variant].name;
+    // (the name of the tile it had first, which programs may look for; now 128 consecutive sites)
     if (precision == LB_RD_FP64) return variant == 0 ? "f64_32x4" : "";
     if ((precision == LB_RD_FP32_BF16DEV || precision == LB_RD_FP32_FP16DEV) && variant >= 0 &&
         variant < lbrd::kHalfVariantCount)

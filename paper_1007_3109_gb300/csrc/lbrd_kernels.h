@@ -215,8 +215,8 @@ bool batch_deep_depth_ok(int K);
 // Default steps per launch of a list of `sites` sites: 6, the deepest two-column
 // form, which moves the state least often; 5 for D2Q9 lists of one species or of
 // fewer than 1.5 M sites, where the rows that fill the levels weigh more (five
-// grids of sides 190 .. 500: 9.1 us per step at K = 5, 9.3 at 6; 9 x 512^2 14.8 /
-// 13.7; 256 x 248^2 94.2 / 82.2).
+// grids of sides 190 .. 500: 8.6 us per step at K = 5, 8.7 at 6; 9 x 512^2 14.9 /
+// 13.6; 256 x 248^2 94.2 / 82.1).
 int batch_deep_default_k(int Q, int S, int64_t sites);
 int64_t batch_deep_plan(int K, int Q, int S, bool v16, DeepItem *items, int n);
 cudaError_t launch_batch_deep(int K, int Q, int S, bool v16, const DeepItem *items, int n, int64_t total_units,

@@ -58,10 +58,11 @@ cudaError_t launch_step_f32_pair(int v, int Q, int S, const StepArgs &a, cudaStr
         // a row staged as soon as level 1 has read the oldest one (one more row in flight;
         // D2Q5: the D2Q9 forms are slower so)
         case 21: return dispatch_pair<6, 4, 3, 1, true, false, true>(Q, S, a, st);
-        // three rows in flight: grids that stay in L2 (512^2 3.30 us per step against 3.37 for the
-        // best K = 5 form, 320 x 256 2.21 / 2.28)
+        // three rows in flight: grids that stay in L2 (320 x 256 2.15 us per step against 2.26 for the
+        // best K = 5 form, 512^2 3.26 / 3.23, 768^2 4.89 / 5.27)
         case 22: return dispatch_pair<4, 4, 3, 1, true, false, true>(Q, S, a, st);
-        // level 4's rows in shared memory (the any-nx form stages late: early, its spills take 1531 x 1021 from 12.4 to 18.7 us)
+        // level 4's rows in shared memory (the any-nx form stages late: early, its spills took 1531 x 1021
+        // from 12.4 to 18.7 us; 11.3 now)
         case 23: return dispatch_pair<6, 8, 2, 1, false, false, true, 8>(Q, S, a, st);
         case 24: return dispatch_pair<6, 4, 2, 2, false, false, false, 8>(Q, S, a, st);
         case 25: return dispatch_pair<6, 8, 2, 1, false, true, false, 8>(Q, S, a, st);

@@ -529,7 +529,8 @@ struct PairKernel {
 // Blocks of four warps for a grid: one per SM where that is estimated to be
 // faster than as many as fit.  Fewer bands fill the levels fewer times, and a
 // warp that has its scheduler to itself walks a row in about 2/3 of the time that
-// each of two take (512^2 at K = 4: 60 bands 3.57 us per step, 121 bands 4.17).
+// each of two take (K = 4, deep4vwp_128_minb1_s6, one block per SM against as many as
+// fit: 512^2 3.26 us per step with 60 bands, 3.70 with 121; 320 x 256 2.15 / 2.82).
 inline unsigned pair_blocks(int K, int64_t nstrips, int64_t ny, unsigned full) {
     const unsigned sms = sm_count();
     if (full <= sms) return full;
