@@ -199,7 +199,9 @@ LB_RD_API int lb_rd_init(lb_rd_handle *h, const double *rho0, int is_device);
  * needed to leave them available.  An untuned handle of more than 65536 sites
  * (tb_depth 0) runs a depth-K variant chosen by its size, with the same
  * results; with track_mass its call ends on a single step, whose mass has the
- * bits of one step per launch. */
+ * bits of one step per launch.  Captured into a CUDA graph, calls of an even
+ * number of steps in all can be replayed: each replay advances the state by
+ * them (the handle's time counts the captured calls only). */
 LB_RD_API int lb_rd_step(lb_rd_handle *h, int64_t nsteps);
 
 /* Current time step t of the handle. */

@@ -332,6 +332,38 @@ LaunchPlan plan_launches(const lb_rd_handle *h, int64_t nsteps, bool single_last
     return p;
 }
 
+// A call that is being captured into a caller's graph takes as many launches as it
+// takes steps, modulo two: the state copies change places with every launch, so a
+// graph of an even number of steps ends where it began and can be replayed, as with
+// one step per launch.  Where the plan's count differs, one of its launches becomes
+// two (or, where no two depths make it up, single steps).
+void match_parity(const lb_rd_handle *h, int64_t nsteps, LaunchPlan &p) {
+    if (((p.bulk + (int64_t)p.tail.size()) ^ nsteps) % 2 == 0) return;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess) {
+        cudaGetLastError();  // the legacy stream beside another stream's capture
+        return;
+    }
+    if (capture == cudaStreamCaptureStatusNone) return;
+    auto ok = [&](int d) { return d == 1 || d == p.K || h->depth_variant[d] >= 0; };
+    auto split = [&](int d) {
+        for (int a = (d + 1) / 2; a < d; ++a)
+            if (ok(a) && ok(d - a)) return std::vector<int>{a, d - a};
+        return d % 2 == 0 ? std::vector<int>(d, 1) : std::vector<int>();
+    };
+    for (size_t i = 0; i < p.tail.size(); ++i) {
+        const std::vector<int> parts = split(p.tail[i]);
+        if (parts.empty()) continue;
+        p.tail.erase(p.tail.begin() + i);
+        p.tail.insert(p.tail.begin() + i, parts.begin(), parts.end());
+        return;
+    }
+    const std::vector<int> parts = p.bulk > 0 ? split(p.K) : std::vector<int>();
+    if (parts.empty()) return;
+    --p.bulk;
+    p.tail.insert(p.tail.begin(), parts.begin(), parts.end());
+}
+
 cudaError_t launch_step(const lb_rd_handle *h, const lbrd::StepArgs &a, int variant) {
     if (h->general) return lbrd::launch_step_general(h->prec == LB_RD_FP64 ? 0 : 1, h->Q, h->S, a, h->stream, variant);
     switch (h->prec) {
@@ -611,7 +643,8 @@ int lb_rd_step(lb_rd_handle *h, int64_t nsteps) {
     // starts from a tuned choice may end on a launch of several steps, whose FP32
     // partial sums are grouped otherwise.)
     const bool mass_last = h->by_size && h->cfg.track_mass;
-    const LaunchPlan plan = plan_launches(h, nsteps, mass_last);
+    LaunchPlan plan = plan_launches(h, nsteps, mass_last);
+    match_parity(h, nsteps, plan);
     const int64_t nl = plan.bulk + (int64_t)plan.tail.size();
     for (int64_t n = 0; n < nl; ++n) {
         const int d = n < plan.bulk ? plan.K : plan.tail[(size_t)(n - plan.bulk)];
