@@ -323,7 +323,9 @@ LB_RD_API int lb_rd_batch_init(lb_rd_batch *b, int32_t idx, const double *rho0, 
  * (lb_rd_batch_set_steps_per_launch) the call runs nsteps / K launches of K
  * steps and one launch of the nsteps % K steps left (a single step if one is
  * left; FP32: the last full launch and those steps as two of nearly equal
- * depth), otherwise its last step is a single step. */
+ * depth), otherwise its last step is a single step.  Captured into a CUDA
+ * graph, a call with depth-K launches of an even number of steps can be
+ * replayed: each replay advances the batch by them. */
 LB_RD_API int lb_rd_batch_step(lb_rd_batch *b, int64_t nsteps);
 
 /* Steps per captured CUDA graph (an even number >= 2), or 0 to launch every

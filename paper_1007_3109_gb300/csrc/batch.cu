@@ -240,17 +240,19 @@ cudaError_t plan_deep(lb_rd_batch *b, int K) {
 }
 
 // Whether a call's last steps can be launched at depths d0 and d1: their
-// descriptors are planned here, before any of the call's launches.  Not while the
-// stream is captured (planning allocates and copies), nor where the memory for them
-// is lacking: the call then runs full launches and the remainder.
+// descriptors are planned here, before any of the call's launches.  Where the memory
+// for them is lacking, the call runs full launches and the remainder.
 bool can_split(lb_rd_batch *b, int d0, int d1) {
-    if (b->deep_units[d0] > 0 && b->deep_units[d1] > 0) return true;
+    if (plan_deep(b, d0) == cudaSuccess && plan_deep(b, d1) == cudaSuccess) return true;
+    cudaGetLastError();  // clear a non-sticky error of the attempt
+    return false;
+}
+
+bool being_captured(cudaStream_t st) {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    const bool ok = cudaStreamIsCapturing(b->stream, &capture) == cudaSuccess &&
-                    capture == cudaStreamCaptureStatusNone && plan_deep(b, d0) == cudaSuccess &&
-                    plan_deep(b, d1) == cudaSuccess;
-    if (!ok) cudaGetLastError();  // clear a non-sticky error of the attempt
-    return ok;
+    if (cudaStreamIsCapturing(st, &capture) == cudaSuccess) return capture != cudaStreamCaptureStatusNone;
+    cudaGetLastError();  // the legacy stream beside another stream's capture
+    return false;
 }
 
 // One depth-K launch of K steps from buffer parity `parity`; emit: it also
@@ -272,6 +274,41 @@ cudaError_t launch_multi(lb_rd_batch *b, int parity) {
     if (uses_tb2(b))
         return lbrd::launch_batch_tb2(b->d_tb[parity], (int)b->cfgs.size(), b->tb_units, b->Q, b->S, b->stream);
     return launch_deep(b, b->steps_per_launch, parity, false);
+}
+
+// The next d steps of a call in one launch.
+cudaError_t advance(lb_rd_batch *b, int d, bool emit) {
+    cudaError_t e = d == 1 ? launch_one(b, b->cur, emit) : launch_deep(b, d, b->cur, emit);
+    if (e) return e;
+    b->cur ^= 1;
+    b->t += d;
+    b->launches++;
+    return cudaSuccess;
+}
+
+// A call of a batch with K steps per launch that is being captured into a caller's
+// graph: planning a depth would allocate and copy, so the steps left after the full
+// launches run one by one unless their depth is planned.  A call of an even number of
+// steps takes an even number of launches (the state copies change places with each),
+// so that its graph can be replayed.
+cudaError_t advance_captured(lb_rd_batch *b, int64_t nsteps) {
+    const int K = b->steps_per_launch;
+    int64_t full = nsteps / K, r = nsteps % K;
+    bool deep = r >= 2 && b->deep_units[r] > 0;
+    int64_t singles = deep ? 0 : r;
+    if (nsteps % 2 == 0 && (full + deep + singles) % 2 != 0) {
+        if (deep) singles = r;
+        deep = false;
+        if ((full + singles) % 2 != 0 && full > 0) {  // K is even
+            --full;
+            singles += K;
+        }
+    }
+    cudaError_t e = cudaSuccess;
+    for (; full > 0 && !e; --full) e = advance(b, K, full == 1 && !deep && singles == 0);
+    if (deep && !e) e = advance(b, (int)r, true);
+    for (; singles > 0 && !e; --singles) e = advance(b, 1, singles == 1);
+    return e;
 }
 
 }  // namespace
@@ -586,25 +623,18 @@ int lb_rd_batch_step(lb_rd_batch *b, int64_t nsteps) {
         // left are two launches of nearly equal depth, since a launch of one or
         // two steps takes about as long as one of four (256 grids of 248^2, us
         // per launch of 1 .. 6 steps: 424, 450, 439, 447, 471, 493)
+        if (being_captured(b->stream)) {
+            cudaError_t e = advance_captured(b, nsteps);
+            return e ? cuda_err(e, "batch step kernel") : LB_RD_OK;
+        }
         const int64_t q = nsteps / K, r = nsteps % K;
         const int tail = r == 0 ? K : (int)r, d0 = (K + tail + 1) / 2;
         const bool even = r > 0 && r < K - 1 && q > 0 && !half_batch(b) && can_split(b, d0, K + tail - d0);
         int rc = run_multi(b, r == 0 || even ? q - 1 : q);
         if (rc) return rc;
-        if (even) {
-            cudaError_t e = launch_deep(b, d0, b->cur, false);
-            if (e) return cuda_err(e, "batch step kernel");
-            b->cur ^= 1;
-            b->t += d0;
-            b->launches++;
-        }
-        const int d = even ? K + tail - d0 : tail;
-        cudaError_t e = d == 1 ? launch_one(b, b->cur, true) : launch_deep(b, d, b->cur, true);
-        if (e) return cuda_err(e, "batch step kernel");
-        b->cur ^= 1;
-        b->t += d;
-        b->launches++;
-        return LB_RD_OK;
+        cudaError_t e = even ? advance(b, d0, false) : cudaSuccess;
+        if (!e) e = advance(b, even ? K + tail - d0 : tail, true);
+        return e ? cuda_err(e, "batch step kernel") : LB_RD_OK;
     }
     int64_t body = nsteps - 1;  // the last step also writes the densities
     if (K >= 2 && body >= K) {
